@@ -53,7 +53,7 @@ def listed():
         dict(name="edge_4096_d2q7", kind="single", lattice="d2q7", width=4096, height=2048, front_row=1024,
              growth="edge", gap=1000.0, front="sinusoidal", steps=20, read="fields"),
         # the FP64 path, the paper's own parameter list with its heavy noise
-        dict(name="paper_512_fp64", kind="single", width=512, height=1024, front_row=64, scale="paper", rate=1e-4,
+        dict(name="paper_512_fp64", kind="single", width=512, height=1024, front_row=64, scale="paper", rate=1e-4, negfix="rescale",
              precision="fp64", steps=10, read="fields"),
         # 256 uneven realisations (widths 256..2048) together, as the roughness statistics need them
         dict(name="ensemble_256_fp32", kind="batch", members="ensemble", n=256, steps=40, read="fields"),
