@@ -139,30 +139,6 @@ __device__ __forceinline__ void momentum7(const R *g, R &jx, R &jy)
     jy = (((g[2] + g[3]) - g[5]) - g[6]) * R(HALF_SQRT3);
 }
 
-// rho and u of copy cur into device arrays of W*H doubles (Eq. 1).
-template <typename S>
-__global__ void k_fields7(SimDev d, int cur, double *rho, double *ux, double *uy)
-{
-    const S *f = (const S *)d.f[cur];
-    const long long total = (long long)d.W * d.H;
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < total;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / d.W), x = (int)(k % d.W);
-        const long long o = (long long)y * d.Wp + x;
-        double g[NQ7];
-#pragma unroll
-        for (int i = 0; i < NQ7; ++i) g[i] = (double)f[i * d.P + o];
-        double r = g[0];
-#pragma unroll
-        for (int i = 1; i < NQ7; ++i) r = r + g[i];
-        double jx, jy;
-        momentum7<double>(g, jx, jy);
-        rho[k] = r;
-        ux[k] = r != 0.0 ? jx / r : 0.0;
-        uy[k] = r != 0.0 ? jy / r : 0.0;
-    }
-}
-
 // ===========================================================================
 // Per-node collision (Eqs. 2-4 and App. A step 7) on seven directions.
 

@@ -875,29 +875,4 @@ __device__ __forceinline__ int division_record(const SimDev &d, int e, uint32_t 
     return owner;
 }
 
-// rho and u of copy `cur` into device arrays of W*H doubles (Eq. 1).
-template <typename S>
-__global__ void k_fields(SimDev d, int cur, double *rho, double *ux, double *uy)
-{
-    const Pop<S> pc(d);
-    const S *f = (const S *)d.f[cur];
-    const long long total = (long long)d.W * d.H;
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < total;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / d.W), x = (int)(k % d.W);
-        const long long o = (long long)y * d.Wp + x;
-        double g[NQ];
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) g[i] = (double)pc.ld(f[i * d.P + o], i);
-        double r = g[0];
-#pragma unroll
-        for (int i = 1; i < NQ; ++i) r = r + g[i];
-        const double jx = ((((g[1] - g[3]) + g[5]) - g[6]) - g[7]) + g[8];
-        const double jy = ((((g[2] - g[4]) + g[5]) + g[6]) - g[7]) - g[8];
-        rho[k] = r;
-        ux[k] = r != 0.0 ? jx / r : 0.0;
-        uy[k] = r != 0.0 ? jy / r : 0.0;
-    }
-}
-
 } // namespace lbm

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "lbm_d2q7.cuh"
+#include "lbm_fields.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_plan.cuh"
 
@@ -45,8 +46,7 @@ struct Launch {
     }
     static cudaError_t fields(const SimDev &d, int cur, double *rho, double *ux, double *uy, cudaStream_t s)
     {
-        k_fields<S><<<4 * 152, 256, 0, s>>>(d, cur, rho, ux, uy);
-        return cudaGetLastError();
+        return launch_fields<S, Lat9>(d, cur, rho, ux, uy, s);
     }
     static cudaError_t batch_inject(const SimDev *ds, int nslots, int grid, cudaStream_t s)
     {
@@ -127,8 +127,7 @@ struct Launch7 {
     }
     static cudaError_t fields(const SimDev &d, int cur, double *rho, double *ux, double *uy, cudaStream_t s)
     {
-        k_fields7<S><<<4 * 152, 256, 0, s>>>(d, cur, rho, ux, uy);
-        return cudaGetLastError();
+        return launch_fields<S, Lat7>(d, cur, rho, ux, uy, s);
     }
     static cudaError_t batch_inject(const SimDev *ds, int nslots, int grid, cudaStream_t s)
     {
