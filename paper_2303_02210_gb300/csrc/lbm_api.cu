@@ -118,7 +118,7 @@ struct Layout {
     long long P;
     int elem;
     uint64_t off_f0, off_f1, off_mask, off_heights, off_rows0, off_sc, off_htab, off_hlist, off_evk,
-        off_evc, off_rown, off_rk, off_roff, off_bcnt, off_bucket, off_pl64, off_pl32, total;
+        off_evc, off_rown, off_rec, off_bcnt, off_bucket, off_pl64, off_pl32, off_xch, total;
 };
 
 Layout make_layout(const lbm_params_t &p)
@@ -157,13 +157,13 @@ Layout make_layout(const lbm_params_t &p)
     L.off_evk = o; o = align256(o + (uint64_t)L.ns_max * 8u);
     L.off_evc = o; o = align256(o + (uint64_t)L.ns_max * 8u);
     L.off_rown = o; o = align256(o + (uint64_t)L.ns_max * 4u);
-    L.off_rk = o; o = align256(o + (uint64_t)L.ns_max * 4u);
-    L.off_roff = o; o = align256(o + (uint64_t)L.ns_max * 8u);
+    L.off_rec = o; o = align256(o + (uint64_t)L.ns_max * 8u);
     L.off_bcnt = o; o = align256(o + (uint64_t)kTmaMaxCtas * 4u);
-    L.off_bucket = o; o = align256(o + (uint64_t)kTmaMaxCtas * kBucketCap * 4u);
+    L.off_bucket = o; o = align256(o + (uint64_t)kTmaMaxCtas * kBucketCap * 8u);
     // planner partials: S1, S2, frozen mass (int64); top, low, two count buffers (int32)
     L.off_pl64 = o; o = align256(o + (uint64_t)kPlanMaxBlocks * 3u * 8u);
     L.off_pl32 = o; o = align256(o + (uint64_t)kPlanMaxBlocks * 4u * 4u);
+    L.off_xch = o; o = align256(o + kXchBytes); // exchanges of a launch of many steps
     L.total = o;
     return L;
 }
@@ -228,6 +228,29 @@ void front_rows(const lbm_params_t &p, std::vector<int32_t> &rows)
     }
 }
 
+// Whether steps run many to a launch (lbm_steps.cuh) rather than as two
+// launches each: while the step's fixed cost counts. By the nodes of the
+// initial active window (rows0: its front), us per step in one launch
+// against two launches: FP32 27 against 33 or less at 0.5M nodes, 44 / 47 at
+// 2.1M, 70.0 / 71.5 at 4.2M, 118.6 / 117.2 at 8.4M (a lone update then has
+// fewer spills and the planner's share is small); 16 bits, which are bound by
+// their instructions, 43.4 / 45.7 at 2.1M, 73.2 / 72.3 at 4.2M, 118.4 /
+// 114.0 at 8.4M; D2Q7 105.6 / 109.6 at 8.4M still.
+bool fused_pays(const lbm_params_t &p, const std::vector<int32_t> &rows0)
+{
+    if (p.lattice == LBM_D2Q7) return true;
+    long long top = 0, sum = 0;
+    for (int32_t r : rows0) {
+        top = std::max<long long>(top, r);
+        sum += r;
+    }
+    long long rear = 0;
+    if (p.wall_mode == LBM_WALL_ADVANCE)
+        rear = (long long)std::max(0.0, std::floor((double)sum / p.width - p.wall_min_gap));
+    const long long nodes = (std::min<long long>(p.height, top + 2) - rear) * p.width;
+    return nodes <= (p.precision == LBM_FP32 ? 6ll << 20 : 4ll << 20);
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no
 // link-time dependency on the driver library).
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
@@ -285,6 +308,7 @@ struct lbm_sim {
     int64_t launches;
     // TMA-staged update (FP32, walls in y)
     bool use_tma;
+    bool fused; // many steps in one launch (update_kernel 0)
     int tma_grid, tma_variant;
     CUtensorMap maps[4]; // loads from copy 0, 1; stores into copy 0, 1 (variants that store in bulk)
     // kernel timing
@@ -446,16 +470,16 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
     d.ev_key = (uint32_t *)(base + L.off_evk);
     d.ev_count = (int32_t *)(base + L.off_evc);
     d.rec_owner = (int *)(base + L.off_rown);
-    d.rec_k = (int *)(base + L.off_rk);
-    d.rec_off = (int *)(base + L.off_roff);
+    d.rec = (unsigned long long *)(base + L.off_rec);
     d.bucket_cnt = (int *)(base + L.off_bcnt);
-    d.bucket = (int *)(base + L.off_bucket);
+    d.bucket = (unsigned long long *)(base + L.off_bucket);
     d.pl_s1 = (long long *)(base + L.off_pl64);
     d.pl_s2 = d.pl_s1 + kPlanMaxBlocks;
     d.pl_mass = d.pl_s2 + kPlanMaxBlocks;
     d.pl_top = (int *)(base + L.off_pl32);
     d.pl_low = d.pl_top + kPlanMaxBlocks;
     d.pl_cnt = d.pl_low + kPlanMaxBlocks; // two buffers
+    d.xch = (unsigned long long *)(base + L.off_xch);
     d.W = p->width;
     d.H = p->height;
     d.Wp = L.Wp;
@@ -530,7 +554,9 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
         delete s;
         return LBM_ERR_CUDA;
     }
-    s->use_tma = false;
+    std::vector<int32_t> rows;
+    front_rows(*p, rows);
+    s->use_tma = s->fused = false;
     s->tma_grid = nsm;
     // staged update variant (KernelTable::tma_info): "tma" 0 (two-row tiles),
     // "tma1" 1 (four-row tiles), "tma_st" 2 (two-row tiles stored in bulk,
@@ -590,6 +616,8 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
             s->use_tma = false;
             d.inject_in_update = 0;
         }
+        s->fused = s->use_tma && p->update_kernel == 0 && s->kt->tma_steps && fused_pays(*p, rows) &&
+                   s->kt->tma_steps(d, nullptr, variant, 0, s->stream) == cudaSuccess;
         if (!ok && p->update_kernel >= 2 && p->update_kernel != 5) {
             if (s->own_arena) cudaFree(s->arena);
             delete s;
@@ -604,8 +632,6 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
         // the division table starts empty (every entry all ones)
         e = cudaMemsetAsync(d.htab, 0xFF, (size_t)L.hcap * 8u, s->stream);
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
-        std::vector<int32_t> rows;
-        front_rows(*p, rows);
         e = cudaMemcpyAsync(d.rows0, rows.data(), sizeof(int32_t) * rows.size(), cudaMemcpyHostToDevice, s->stream);
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = s->kt->fill(d, s->stream)) != cudaSuccess) { rc = cuda_fail(e); break; }
@@ -646,6 +672,19 @@ int lbm_step(lbm_sim *s, int64_t nsteps)
 {
     if (!s || nsteps < 0) return LBM_ERR_INVALID_ARG;
     USE_DEVICE(s);
+    if (s->fused && !s->timing) {
+        // (launches of at most kStepsPerLaunch steps: work on other streams
+        // gets its turn between them)
+        for (int64_t left = nsteps; left > 0;) {
+            const int n = (int)std::min<int64_t>(left, kStepsPerLaunch);
+            CK(s->kt->tma_steps(s->d, s->maps, s->tma_variant, n, s->stream));
+            ++s->launches;
+            s->cur ^= n & 1;
+            s->step += n;
+            left -= n;
+        }
+        return LBM_OK;
+    }
     for (int64_t k = 0; k < nsteps; ++k) {
         const bool timed = s->timing && (s->timing_count++ % s->timing_stride) == 0 &&
                            s->ev_used + 2 <= (int64_t)s->ev.size();
@@ -734,6 +773,8 @@ int lbm_clear_status(lbm_sim *s)
     // next planner needs)
     CK(cudaMemsetAsync(&s->d.sc->bar_ctr, 0, sizeof(unsigned long long), s->stream));
     CK(cudaMemsetAsync(s->d.htab, 0xFF, (size_t)s->L.hcap * 8u, s->stream));
+    CK(cudaMemsetAsync(s->d.xch, 0, kXchBytes, s->stream)); // (a step may be run again under the same number)
+    CK(cudaMemsetAsync(s->d.ev_count, 0, (size_t)s->L.ns_max * 8u, s->stream)); // (zero beyond the current selections)
     return LBM_OK;
 }
 

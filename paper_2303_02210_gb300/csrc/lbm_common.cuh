@@ -44,6 +44,20 @@ __host__ __device__ __forceinline__ int key_x(uint32_t k) { return (int)((k >> 2
 __host__ __device__ __forceinline__ int key_y(uint32_t k) { return (int)(k >> 17); }
 __host__ __device__ __forceinline__ int key_pair(uint32_t k) { return (int)(k & 3u); }
 
+// A division's record in its update CTA's bucket: draw rank (< 2^24), the
+// tile's index among the CTA's tiles (at most 2^30 nodes in tiles of 256 over
+// at least an eighth as many CTAs or all that fit: < 2^14) and the two staged
+// offsets (< 2^13).
+__host__ __device__ __forceinline__ unsigned long long pack_record(int rank, int k, int off0, int off1)
+{
+    return (unsigned long long)(uint32_t)rank << 40 | (unsigned long long)(uint32_t)k << 26 |
+           (unsigned long long)(uint32_t)off0 << 13 | (uint32_t)off1;
+}
+__host__ __device__ __forceinline__ int rec_rank(unsigned long long r) { return (int)(r >> 40); }
+__host__ __device__ __forceinline__ int rec_tile(unsigned long long r) { return (int)(r >> 26) & 0x3FFF; }
+__host__ __device__ __forceinline__ int rec_off0(unsigned long long r) { return (int)(r >> 13) & 0x1FFF; }
+__host__ __device__ __forceinline__ int rec_off1(unsigned long long r) { return (int)r & 0x1FFF; }
+
 // Fixed-point unit of the exact mass sums: 2^-24 per count.
 constexpr double kFixScale = 16777216.0;
 constexpr double kFixInv = 5.9604644775390625e-08;
@@ -149,6 +163,13 @@ struct DevScalars {
     // the latest selection): copied from pend_cand by the batched injection
     // launch, read by the batched planner launches that follow it
     long long plan_work;
+    // a launch of many steps (lbm_steps.cuh): CTAs that finished their update
+    // and planner CTAs that finished, since the launch began (each counter on
+    // a line of its own; zero between launches); set when a wait ran out; CTAs
+    // that left
+    unsigned long long pad4[16], st_up, pad5[15], st_done, pad6[15];
+    int st_quit;
+    unsigned int st_exit;
 };
 enum { WAIT_TEST_COPIES = 1, WAIT_TEST_BARRIER = 2 };
 // Default budget of the bounded waits: about two seconds at 2 GHz.
@@ -184,15 +205,14 @@ struct SimDev {
     int upd_ctas;         // CTAs of the TMA-staged update kernel (tiles dealt round-robin)
     uint32_t upd_magic;   // ceil(2^32 / upd_ctas), upd_ctas >= 2: tile / upd_ctas = umulhi(tile, magic)
     int upd_tyl2;         // log2 of the rows per tile of the TMA-staged update
-    int *rec_owner;       // per division (selector order): owning CTA of its tile,
-    int *rec_k;           // the tile's index among that CTA's tiles,
-    int *rec_off;         // and the two pre-stream slots' offsets in the staged box
-                          // (the amount is ev_count * rho_cell / 2)
+    int *rec_owner;       // per division (draw rank): owning CTA of its tile (-1: a repeat)
+    unsigned long long *rec; // and its record (pack_record; the amount is ev_count * rho_cell / 2)
     int *bucket_cnt;      // divisions per CTA of the TMA-staged update (kTmaMaxCtas)
-    int *bucket;          // their record indices, kBucketCap per CTA
+    unsigned long long *bucket; // their records (pack_record), kBucketCap per CTA
     // per-block partials of the fused planner (kPlanMaxBlocks each)
     long long *pl_s1, *pl_s2, *pl_mass;
     int *pl_top, *pl_low, *pl_cnt;
+    unsigned long long *xch; // the exchanges of a launch of many steps (lbm_steps.cuh)
     int plan_grid;        // blocks of the fused planner (all co-resident)
     // the same constants rounded to float once on the host, so that no kernel
     // evaluates double arithmetic per node (the FP64 pipe is narrow)
@@ -247,6 +267,10 @@ struct KernelTable {
     // pdl: launch as a programmatic dependent of the preceding kernel.
     cudaError_t (*tma_prepare)(const SimDev &, int variant);
     cudaError_t (*tma_update)(const SimDev &, const CUtensorMap *maps, int variant, bool pdl, cudaStream_t);
+    // `steps` whole steps in one cooperative launch (lbm_steps.cuh); with
+    // maps null, only reports whether the launch fits the device
+    // (cudaErrorCooperativeLaunchTooLarge if not)
+    cudaError_t (*tma_steps)(const SimDev &, const CUtensorMap *maps, int variant, int steps, cudaStream_t);
     // a staged variant's geometry: rows of one bulk copy's box, rows per
     // tile, CTAs per SM; 0 for a variant the table has, 1 for one that also
     // stores in bulk, -1 for none
@@ -285,6 +309,12 @@ constexpr int kTmaBoxX = 128;
 constexpr int kTmaMaxCtas = 2048; // the reciprocal above is exact for tile * upd_ctas < 2^32
 constexpr int kBucketCap = 256;    // division records listed per update CTA (more: full scan)
 constexpr int kPlanMaxBlocks = 1024;
+// A launch of many steps (lbm_steps.cuh): planner CTAs, exchanged words of 8
+// bytes per CTA, and steps per launch.
+constexpr int kStepMaxPlan = 256;
+constexpr int kXch = 8;
+constexpr size_t kXchBytes = (size_t)kStepMaxPlan * kXch * 8u;
+constexpr int kStepsPerLaunch = 64;
 // The TMA-staged batched update: members one launch takes (its shared-memory
 // tables) and CTAs per SM.
 constexpr int kTmaBatchMaxSims = 256;

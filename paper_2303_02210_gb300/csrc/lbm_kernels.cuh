@@ -125,6 +125,15 @@ __device__ __forceinline__ long long warp_sum_ll(long long v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+// The same for v >= 0 by three 32-bit reductions (21 bits of v each; the sum
+// modulo 2^63).
+__device__ __forceinline__ long long warp_sum_u63(long long v)
+{
+    const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x1FFFFFu);
+    const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 21) & 0x1FFFFFu);
+    const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 42));
+    return (long long)(((unsigned long long)c << 42) + ((unsigned long long)b << 21) + a);
+}
 __device__ __forceinline__ double warp_sum_d(double v)
 {
 #pragma unroll
@@ -169,6 +178,10 @@ __device__ __forceinline__ long long pull_slot(const SimDev &d, int y_r, int x, 
 // the neighbour of (x, y) along 2 is (x + (y & 1), y + 1).
 struct Lat9 {
     static constexpr int Q = 9;
+    // source of direction q at (x, y), away from walls
+    __device__ static int dx(int q, int) { return -ex(q); }
+    __device__ static int dy(int q) { return -ey(q); }
+    __device__ static int op(int q) { return opp(q); }
     __device__ static long long slot(const SimDev &d, int y_r, int x, int y, int q)
     {
         return pull_slot(d, y_r, x, y, q);
@@ -189,6 +202,9 @@ __host__ __device__ constexpr int src7_dy(int q) { return q == 2 || q == 3 ? -1 
 
 struct Lat7 {
     static constexpr int Q = 7;
+    __device__ static int dx(int q, int y) { return src7_dx(q, y & 1); }
+    __device__ static int dy(int q) { return src7_dy(q); }
+    __device__ static int op(int q) { return opp7(q); }
     __device__ static long long slot(const SimDev &d, int y_r, int x, int y, int q)
     {
         int ys = y + src7_dy(q);
@@ -779,12 +795,26 @@ __device__ __forceinline__ arith_t<S> rho_star(const SimDev &d, const S *f, int 
 {
     using R = arith_t<S>;
     const Pop<S> pc(d);
-    long long o[LT::Q];
-#pragma unroll
-    for (int q = 0; q < LT::Q; ++q) o[q] = LT::slot(d, y_r, x, y, q);
     R v[LT::Q];
+    if (!d.y_periodic) {
+        // the ghost columns make every source a fixed offset: no wrap, and
+        // across a wall the node's own opposite population by selection (the
+        // planner's time is the length of its instruction chain)
+        const S *b = f + (long long)y * d.Wp + x;
+        const bool lo = y <= y_r, hi = y + 1 >= d.H;
 #pragma unroll
-    for (int q = 0; q < LT::Q; ++q) v[q] = pc.ld(f[o[q]], q);
+        for (int q = 0; q < LT::Q; ++q) {
+            const bool own = LT::dy(q) < 0 ? lo : (LT::dy(q) > 0 ? hi : false);
+            const long long o = own ? LT::op(q) * d.P : q * d.P + (LT::dy(q) * d.Wp + LT::dx(q, y));
+            v[q] = pc.ld(b[o], q);
+        }
+    } else {
+        long long o[LT::Q];
+#pragma unroll
+        for (int q = 0; q < LT::Q; ++q) o[q] = LT::slot(d, y_r, x, y, q);
+#pragma unroll
+        for (int q = 0; q < LT::Q; ++q) v[q] = pc.ld(f[o[q]], q);
+    }
     R r = v[0];
 #pragma unroll
     for (int q = 1; q < LT::Q; ++q) r = r + v[q];
@@ -796,11 +826,10 @@ struct Candidate {
     uint32_t u; // acceptance uniform word (density-dependent growth)
 };
 
+// The candidate that the Philox block r of its counter draws.
 template <typename LT = Lat9>
-__device__ __forceinline__ Candidate draw_candidate(const SimDev &d, long long k, uint32_t t, int ylo,
-                                                    unsigned long long nwin)
+__device__ __forceinline__ Candidate candidate_of(const SimDev &d, const u32x4 &r, int ylo, unsigned long long nwin)
 {
-    const u32x4 r = philox4x32_10(u32x4{(uint32_t)k, t, STREAM_PROLIF, d.sim}, d.pk);
     // node = ylo W + floor(r.x nwin / 2^32); nwin <= W H < 2^30, so the offset
     // in the window splits into row and column in 32-bit arithmetic
     const uint32_t idx = (uint32_t)(((unsigned long long)r.x * nwin) >> 32);
@@ -810,6 +839,13 @@ __device__ __forceinline__ Candidate draw_candidate(const SimDev &d, long long k
     c.pair = LT::pair_of(r.y);
     c.u = r.z;
     return c;
+}
+
+template <typename LT = Lat9>
+__device__ __forceinline__ Candidate draw_candidate(const SimDev &d, long long k, uint32_t t, int ylo,
+                                                    unsigned long long nwin)
+{
+    return candidate_of<LT>(d, philox4x32_10(u32x4{(uint32_t)k, t, STREAM_PROLIF, d.sim}, d.pk), ylo, nwin);
 }
 
 constexpr uint32_t EMPTY_KEY = 0xFFFFFFFFu;
@@ -850,9 +886,9 @@ __device__ __forceinline__ int table_insert(const EventTable &tb, uint32_t key, 
 // ((kTmaBoxX + 8) x (2^upd_tyl2 + 2) x 9 with the tile at column 4, row 1):
 // the source (x - ex_q, y - ey_q) unwrapped in x (the box holds the ghost
 // columns -1 and W), or across a wall the node's own population opp(q).
-// Returns the owner CTA.
+// Returns the owner CTA and the packed record.
 template <typename R>
-__device__ __forceinline__ int division_record(const SimDev &d, int e, uint32_t key, int y_r)
+__device__ __forceinline__ int division_record(const SimDev &d, int e, uint32_t key, int y_r, unsigned long long *rec)
 {
     constexpr int LX = kTmaBoxX + 8;
     const int TY = 1 << d.upd_tyl2, PL = (TY + 2) * LX;
@@ -863,15 +899,15 @@ __device__ __forceinline__ int division_record(const SimDev &d, int e, uint32_t 
     const uint32_t q = __umulhi(tile, d.upd_magic);
     const int x0 = tx * kTmaBoxX, y0 = y_r + ty * TY;
     const int owner = (int)(tile - q * (uint32_t)d.upd_ctas);
-    d.rec_owner[e] = owner;
-    d.rec_k[e] = (int)q;
+    int off[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int qd = h == 0 ? pair_a(p) : pair_b(p);
         const int ys = y - ey(qd);
-        d.rec_off[2 * e + h] = (ys < y_r || ys >= d.H) ? opp(qd) * PL + (y - y0 + 1) * LX + (x - x0 + 4)
+        off[h] = (ys < y_r || ys >= d.H) ? opp(qd) * PL + (y - y0 + 1) * LX + (x - x0 + 4)
                                                        : qd * PL + (ys - y0 + 1) * LX + (x - ex(qd) - x0 + 4);
     }
+    *rec = pack_record(e, (int)q, off[0], off[1]);
     return owner;
 }
 

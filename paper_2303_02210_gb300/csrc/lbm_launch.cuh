@@ -75,6 +75,8 @@ template <typename S>
 constexpr KernelTable make_table(cudaError_t (*tma_prepare)(const SimDev &, int) = nullptr,
                                  cudaError_t (*tma_update)(const SimDev &, const CUtensorMap *, int, bool,
                                                            cudaStream_t) = nullptr,
+                                 cudaError_t (*tma_steps)(const SimDev &, const CUtensorMap *, int, int,
+                                                          cudaStream_t) = nullptr,
                                  int (*tma_info)(int, int *, int *, int *) = nullptr,
                                  cudaError_t (*batch_update_tma)(const SimDev *, const MemberConst *,
                                                                  const CUtensorMap *, int, int, int, int,
@@ -84,7 +86,8 @@ constexpr KernelTable make_table(cudaError_t (*tma_prepare)(const SimDev &, int)
                        &Launch<S>::scan,     &Launch<S>::plan,          &Launch<S>::inject,
                        &Launch<S>::update,
                        &Launch<S>::fields,   &plan_blocks_per_sm<S>,    &Launch<S>::update_blocks_per_sm,
-                       Launch<S>::UPD_TPB,   tma_prepare,               tma_update,        tma_info,
+                       Launch<S>::UPD_TPB,   tma_prepare,               tma_update,        tma_steps,
+                       tma_info,
                        &Launch<S>::batch_inject, &Launch<S>::batch_update, &Launch<S>::batch_plan,
                        batch_update_tma};
 }
@@ -159,13 +162,16 @@ template <typename S>
 constexpr KernelTable make_table7(cudaError_t (*tma_prepare)(const SimDev &, int) = nullptr,
                                   cudaError_t (*tma_update)(const SimDev &, const CUtensorMap *, int, bool,
                                                             cudaStream_t) = nullptr,
+                                  cudaError_t (*tma_steps)(const SimDev &, const CUtensorMap *, int, int,
+                                                           cudaStream_t) = nullptr,
                                   int (*tma_info)(int, int *, int *, int *) = nullptr)
 {
     return KernelTable{(int)sizeof(S),         &Launch7<S>::fill,          &Launch7<S>::ghosts,
                        &Launch7<S>::scan,      &Launch7<S>::plan,          &Launch7<S>::inject,
                        &Launch7<S>::update,    &Launch7<S>::fields,        &plan_blocks_per_sm<S, Lat7>,
                        &Launch7<S>::update_blocks_per_sm,
-                       Launch7<S>::UPD_TPB,    tma_prepare,                tma_update,        tma_info,
+                       Launch7<S>::UPD_TPB,    tma_prepare,                tma_update,        tma_steps,
+                       tma_info,
                        &Launch7<S>::batch_inject, &Launch7<S>::batch_update, &Launch7<S>::batch_plan,
                        nullptr};
 }

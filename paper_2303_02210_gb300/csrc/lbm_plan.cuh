@@ -117,33 +117,36 @@ __device__ __forceinline__ int plan_block_exscan(int v, int *total, int *s_i)
 
 // The division of draw rank `rank`: merged in the table keyed by (node,
 // pair) and counted at the rank of the pair's first draw (ev_count of a
-// repeat stays 0; the counts were zeroed for this selection). The rank's list
+// repeat stays 0; the counts were zero before this selection). The rank's list
 // entry is the table slot if this draw was the first of its (node, pair),
-// else -1. For the TMA-staged update, a first draw also gets its record and
-// a place in its owner CTA's bucket (y_r: the rear wall of the coming step).
+// else -1. For the TMA-staged update, every draw also gets its record and a
+// place in its owner CTA's bucket (y_r: the rear wall of the coming step),
+// a repeat too (its amount is then 0 and the update skips it): the bucket's
+// atomic does not wait for the table's.
 template <typename R, typename LT = Lat9>
 __device__ __forceinline__ void plan_select(const SimDev &d, uint32_t key, int rank, size_t buf, int y_r)
 {
     EventTable tb;
     tb.e = d.htab;
     tb.mask = (unsigned)d.hcap - 1u;
+    int at = kBucketCap, owner = 0;
+    unsigned long long rec = 0ull;
+    if (d.inject_in_update) { // records for the TMA-staged update
+        if constexpr (LT::Q == 9)
+            owner = division_record<R>(d, rank, key, y_r, &rec);
+        else
+            owner = division_record7(d, rank, key, y_r, &rec);
+        at = atomicAdd(&d.bucket_cnt[owner], 1);
+    }
     int first;
     const int slot = table_insert(tb, key, rank, &first);
     d.hlist[rank] = slot;
     d.ev_key[buf + rank] = key;
     if (first >= 0) atomicAdd(&d.ev_count[buf + first], 1);
-    if (d.inject_in_update) { // records for the TMA-staged update
-        if (slot >= 0) {
-            int owner;
-            if constexpr (LT::Q == 9)
-                owner = division_record<R>(d, rank, key, y_r);
-            else
-                owner = division_record7(d, rank, key, y_r);
-            const int at = atomicAdd(&d.bucket_cnt[owner], 1);
-            if (at < kBucketCap) d.bucket[owner * kBucketCap + at] = rank;
-        } else {
-            d.rec_owner[rank] = -1;
-        }
+    if (d.inject_in_update) {
+        if (at < kBucketCap) d.bucket[(size_t)owner * kBucketCap + at] = rec;
+        d.rec[rank] = rec;
+        d.rec_owner[rank] = slot >= 0 ? owner : -1;
     }
 }
 
@@ -216,6 +219,7 @@ __device__ __forceinline__ void plan_body(const SimDev &d, int init, int G, int 
     const long long mass_acc = (long long)sc->mass_accum;
     const double carry_in = init ? sc->carry : sc->pend_carry;
     const double ratio_in = sc->acc_ratio;
+    const int nev_prev = sc->n_events, nsel_prev = sc->rec_n;
     const bool grow = d.growth_mode != GROW_NONE;
     const long long wait_budget = sc->wait_budget > 0 ? sc->wait_budget : kWaitBudget;
     const int wait_extra = (sc->wait_test & WAIT_TEST_BARRIER) ? 1 : 0;
@@ -461,7 +465,13 @@ __device__ __forceinline__ void plan_body(const SimDev &d, int init, int G, int 
     const size_t buf = (size_t)(tn & 1u) * (size_t)d.ns_max; // event list of step tn
     // counts of this selection start at zero (the selection below adds to
     // them after the next grid barrier)
-    for (long long r = (long long)blk * PLAN_NT + tid; r < ns; r += (long long)G * PLAN_NT) d.ev_count[buf + r] = 0;
+    // (and as far as the list's previous selections went, so that all counts
+    // beyond this selection are zero: a launch of many steps relies on it)
+    {
+        const long long nz = max(ns, (long long)max(nev_prev, nsel_prev));
+        for (long long r = (long long)blk * PLAN_NT + tid; r < nz; r += (long long)G * PLAN_NT)
+            d.ev_count[buf + r] = 0;
+    }
 
     // ---- C/D: candidates in draw order, the first n_s accepted, merged
     long long acc = 0; // accepted candidates so far (all blocks agree)

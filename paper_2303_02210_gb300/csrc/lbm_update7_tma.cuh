@@ -145,54 +145,36 @@ __device__ __forceinline__ void store_nodes7(float *o, long long P, const float 
     }
 }
 
-template <int TY, int STAGES, int CTAS, bool NOISE>
-__global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
-    k_update7_tma(SimDev d, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1)
+// One update: the CTA's tiles of the step that the device scalars hold.
+// Returns whether a wait of this thread gave up.
+template <int TY, int STAGES, bool NOISE, bool FUSED>
+__device__ __forceinline__ bool update7_tma_step(const SimDev &d, const CUtensorMap *tm0, const CUtensorMap *tm1,
+                                                 float *s_in, uint64_t *full, uint64_t *empty, int *ev_k,
+                                                 unsigned *kflag, int &s_abort, int &s_nev, TmaStep &st)
 {
     using G = Tma7Geom<TY>;
-    constexpr int NT = G::NT, PLANE = G::PLANE, WARPS = NT / 32;
-    extern __shared__ __align__(128) float smem_f[];
-    // stages on a 128-byte boundary (offset from the array itself)
-    float *s_in = smem_f + ((128u - (smem_u32(smem_f) & 127u)) & 127u) / 4u;
-    uint64_t *full = reinterpret_cast<uint64_t *>(s_in + STAGES * G::STRIDE);
-    uint64_t *empty = full + STAGES;
-    // divisions of this CTA's tiles: local tile index, two staged offsets, amount
-    int *ev_k = reinterpret_cast<int *>(empty + STAGES);
+    constexpr int NT = G::NT, PLANE = G::PLANE;
     int *ev_off = ev_k + TMA_EV_CAP;
     float *ev_add = reinterpret_cast<float *>(ev_off + 2 * TMA_EV_CAP);
-    unsigned *kflag = reinterpret_cast<unsigned *>(ev_add + TMA_EV_CAP); // tiles with divisions
-    __shared__ int s_abort, s_nev;
-
     const int W = d.W, H = d.H, Wp = d.Wp;
     const long long P = d.P;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int half = warp & 1, row = warp >> 1; // column half and row of the tile
-
-    // prologue, which may overlap the end of the kernel before (programmatic
-    // dependent launch): barriers and tensor maps
-    if (tid == 0) {
-        s_abort = 0;
-        s_nev = 0;
-        prefetch_tensormap(&tm0);
-        prefetch_tensormap(&tm1);
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], WARPS);
-        }
-        fence_mbar_init();
-    }
-    if (tid < TMA_KFLAG_WORDS) kflag[tid] = 0u;
-    __syncthreads();
-    grid_dependency_wait();
     const uint32_t t = (uint32_t)d.sc->step;
     // bounded waits: the budget (a failure-detection test shortens it and may
     // withhold the bulk copies, so that the first wait of every thread runs out)
     const long long budget = d.sc->wait_budget > 0 ? d.sc->wait_budget : kWaitBudget;
     const bool withhold = (d.sc->wait_test & WAIT_TEST_COPIES) != 0;
+    st.t = t;
+    st.budget = budget;
+    if (FUSED) {
+        st.extra = (d.sc->wait_test & WAIT_TEST_BARRIER) ? 1 : 0;
+        st.G = step_planners<NT>(d.sc->plan_kc, d.MW, (int)gridDim.x, &st.whole);
+    }
     const int cur = (int)(t & 1u);
-    const CUtensorMap *tm = cur ? &tm1 : &tm0;
-    const float *__restrict__ fin = (const float *)d.f[cur];
-    float *__restrict__ fout = (float *)d.f[cur ^ 1];
+    const CUtensorMap *tm = cur ? tm1 : tm0;
+    const float *fin = (const float *)d.f[cur];
+    float *fout = (float *)d.f[cur ^ 1];
     const int y_r = d.sc->y_r, y_copy = d.sc->y_copy, y_hi = d.sc->y_hi;
 
     // rows the rear wall has just frozen: bring this copy up to date (whole
@@ -211,13 +193,14 @@ __global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
     const int nty = nrows > 0 ? (nrows + TY - 1) / TY : 0;
     const int ntiles = ncx * nty;
     const int Gd = (int)gridDim.x;
+    const int base = st.tiles; // tiles this CTA has staged in the launch's steps before
     const int count = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / Gd + 1 : 0;
     // tile k of this CTA is blockIdx.x + k Gd; its (tx, ty) advance by (Gd % ncx, Gd / ncx)
     const int dtx = Gd % ncx, dty = Gd / ncx;
     // producer state (thread 0): next tile to load and copies issued
     int itx = (int)blockIdx.x % ncx, ity = (int)blockIdx.x / ncx, issued = 0;
     auto issue = [&]() {
-        const int s = issued % STAGES;
+        const int s = (base + issued) % STAGES;
         mbar_arrive_expect_tx(&full[s], G::BYTES);
         tma_load_3d(s_in + s * G::STRIDE, tm, itx * TMA_TX - 4 + kXO, y_r + ity * TY - 1, 0, &full[s]);
         ++issued;
@@ -238,15 +221,18 @@ __global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
     auto amount = [&](int e) {
         return (float)((double)d.ev_count[(size_t)(t & 1u) * (size_t)d.ns_max + (size_t)e] * d.half_cell);
     };
-    const int mine = nev_all > 0 ? d.bucket_cnt[blockIdx.x] : 0;
-    if (mine <= TMA_EV_CAP) { // (the bucket holds kBucketCap >= TMA_EV_CAP records)
-        for (int j = tid; j < mine; j += NT) {
-            const int e = d.bucket[blockIdx.x * kBucketCap + j];
-            const int k = d.rec_k[e];
-            ev_k[j] = k;
-            ev_off[2 * j] = d.rec_off[2 * e];
-            ev_off[2 * j + 1] = d.rec_off[2 * e + 1];
-            ev_add[j] = amount(e);
+    // (one entry per thread, read without waiting for their number)
+    static_assert(NT >= TMA_EV_CAP && kBucketCap >= TMA_EV_CAP, "one bucket entry per thread");
+    const unsigned long long rec = d.inject_in_update && tid < TMA_EV_CAP ? d.bucket[blockIdx.x * kBucketCap + tid] : 0ull;
+    const int in_bucket = d.inject_in_update ? d.bucket_cnt[blockIdx.x] : 0;
+    const int mine = nev_all > 0 ? in_bucket : 0;
+    if (mine <= TMA_EV_CAP) {
+        if (tid < mine) {
+            const int k = rec_tile(rec);
+            ev_k[tid] = k;
+            ev_off[2 * tid] = rec_off0(rec);
+            ev_off[2 * tid + 1] = rec_off1(rec);
+            ev_add[tid] = amount(rec_rank(rec));
             if (k < 32 * TMA_KFLAG_WORDS) atomicOr(&kflag[k >> 5], 1u << (k & 31));
         }
         if (tid == 0) s_nev = mine;
@@ -254,17 +240,31 @@ __global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
         for (int e = tid; e < nev_all; e += NT) {
             if (d.rec_owner[e] != (int)blockIdx.x) continue;
             const int at = atomicAdd(&s_nev, 1);
-            const int k = d.rec_k[e];
+            const unsigned long long r = d.rec[e];
+            const int k = rec_tile(r);
             if (at < TMA_EV_CAP) {
                 ev_k[at] = k;
-                ev_off[2 * at] = d.rec_off[2 * e];
-                ev_off[2 * at + 1] = d.rec_off[2 * e + 1];
+                ev_off[2 * at] = rec_off0(r);
+                ev_off[2 * at + 1] = rec_off1(r);
                 ev_add[at] = amount(e);
             }
             if (k < 32 * TMA_KFLAG_WORDS) atomicOr(&kflag[k >> 5], 1u << (k & 31));
         }
     }
     __syncthreads();
+    if (FUSED) {
+        // this CTA's bucket, its share of the merge table's entries and of the
+        // counts of the selection before the present one are emptied for the
+        // selection that follows this update
+        if (tid == 0 && d.inject_in_update) d.bucket_cnt[blockIdx.x] = 0;
+        const int nsel = d.sc->rec_n, nev = d.sc->n_events;
+        const size_t obuf = (size_t)((t + 1u) & 1u) * (size_t)d.ns_max;
+        for (int r = (int)blockIdx.x * NT + tid; r < nev; r += Gd * NT) d.ev_count[obuf + r] = 0;
+        for (int r = (int)blockIdx.x * NT + tid; r < nsel; r += Gd * NT) {
+            const int slot = d.hlist[r];
+            if (slot >= 0) d.htab[slot] = EMPTY_ENTRY;
+        }
+    }
     const int nev = s_nev;                     // divisions of this CTA
     const bool ev_overflow = nev > TMA_EV_CAP; // then scan the global list per tile
 
@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
     int tx = (int)blockIdx.x % ncx, ty = (int)blockIdx.x / ncx;
 
     for (int k = 0; k < count; ++k) {
-        const int s = k % STAGES;
-        const uint32_t parity = (uint32_t)((k / STAGES) & 1);
+        const int s = (base + k) % STAGES;
+        const uint32_t parity = (uint32_t)(((base + k) / STAGES) & 1);
         const int x0 = tx * TMA_TX, y0 = y_r + ty * TY;
         float *stage = s_in + s * G::STRIDE;
         if (!dead && !mbar_wait_bounded(&full[s], parity, budget)) {
@@ -294,16 +294,16 @@ __global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
         if (has_ev) { // uniform across the CTA
             if (!ev_overflow) {
                 for (int i = tid; i < nev; i += NT)
-                    if (ev_k[i] == k) {
+                    if (ev_k[i] == k && ev_add[i] != 0.0f) { // (0: a repeat)
                         stage[ev_off[2 * i]] = stage[ev_off[2 * i]] + ev_add[i];
                         stage[ev_off[2 * i + 1]] = stage[ev_off[2 * i + 1]] + ev_add[i];
                     }
             } else {
                 for (int e = tid; e < nev_all; e += NT)
-                    if (d.rec_owner[e] == (int)blockIdx.x && d.rec_k[e] == k) {
+                    if (d.rec_owner[e] == (int)blockIdx.x && rec_tile(d.rec[e]) == k) {
                         const float a = amount(e);
-                        stage[d.rec_off[2 * e]] = stage[d.rec_off[2 * e]] + a;
-                        stage[d.rec_off[2 * e + 1]] = stage[d.rec_off[2 * e + 1]] + a;
+                        stage[rec_off0(d.rec[e])] = stage[rec_off0(d.rec[e])] + a;
+                        stage[rec_off1(d.rec[e])] = stage[rec_off1(d.rec[e])] + a;
                     }
             }
             fence_proxy_async_smem(); // before a later bulk copy overwrites them
@@ -447,20 +447,80 @@ __global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
         atomicOr(&d.sc->status, ST_TIMEOUT);
         // let the copies still in flight land before the CTA exits
         for (int k = issued - STAGES > 0 ? issued - STAGES : 0; k < issued; ++k)
-            mbar_wait_bounded(&full[k % STAGES], (uint32_t)((k / STAGES) & 1), kWaitBudget);
+            mbar_wait_bounded(&full[(base + k) % STAGES], (uint32_t)(((base + k) / STAGES) & 1), kWaitBudget);
     }
-    mass = warp_sum_ll(mass);
-    maxrow = warp_max_i(maxrow);
-    const double clipd = warp_sum_d((double)clip);
+    mass = warp_sum_u63(mass);
+    maxrow = __reduce_max_sync(0xffffffffu, maxrow);
+    const double clipd = __any_sync(0xffffffffu, clip != 0.0f) ? warp_sum_d((double)clip) : 0.0;
     if (lane == 0) {
         if (mass != 0) atomicAdd(&d.sc->mass_accum, (unsigned long long)mass);
         if (maxrow >= 0) atomicMax(&d.sc->maxmass_accum, maxrow);
         if (clipd != 0.0) atomicAdd(&d.sc->clip_mass, clipd);
     }
+    st.tiles = base + count;
+    return dead;
+}
+
+// FUSED: `nsteps` whole steps in this launch (lbm_steps.cuh), else one update.
+template <int TY, int STAGES, int CTAS, bool NOISE, bool FUSED>
+__global__ void __launch_bounds__(Tma7Geom<TY>::NT, CTAS)
+    k_update7_tma(SimDev d, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
+                  int nsteps)
+{
+    using G = Tma7Geom<TY>;
+    constexpr int NT = G::NT, WARPS = NT / 32;
+    extern __shared__ __align__(128) float smem_f[];
+    // stages on a 128-byte boundary (offset from the array itself)
+    float *s_in = smem_f + ((128u - (smem_u32(smem_f) & 127u)) & 127u) / 4u;
+    uint64_t *full = reinterpret_cast<uint64_t *>(s_in + STAGES * G::STRIDE);
+    uint64_t *empty = full + STAGES;
+    // divisions of this CTA's tiles: local tile index, two staged offsets, amount
+    int *ev_k = reinterpret_cast<int *>(empty + STAGES);
+    unsigned *kflag = reinterpret_cast<unsigned *>(ev_k + 4 * TMA_EV_CAP); // tiles with divisions
+    __shared__ int s_abort, s_nev;
+    const int tid = threadIdx.x;
+
+    // prologue, which may overlap the end of the kernel before (programmatic
+    // dependent launch): barriers and tensor maps
+    if (tid == 0) {
+        s_abort = 0;
+        s_nev = 0;
+        prefetch_tensormap(&tm0);
+        prefetch_tensormap(&tm1);
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], WARPS);
+        }
+        fence_mbar_init();
+    }
+    if (tid < TMA_KFLAG_WORDS) kflag[tid] = 0u;
+    __syncthreads();
+    grid_dependency_wait();
+    TmaStep st;
+    st.tiles = 0;
+    if constexpr (!FUSED) {
+        update7_tma_step<TY, STAGES, NOISE, false>(d, &tm0, &tm1, s_in, full, empty, ev_k, kflag, s_abort, s_nev, st);
+    } else {
+        using Scratch = StepScratch<NT>;
+        static_assert(sizeof(Scratch) <= (size_t)STAGES * G::STRIDE * 4, "the planner's room");
+        const long long after = d.sc->step + nsteps;
+        unsigned long long planned = 0;
+        for (int it = 0; it < nsteps; ++it) {
+            const bool gave_up = update7_tma_step<TY, STAGES, NOISE, true>(d, &tm0, &tm1, s_in, full, empty, ev_k,
+                                                                           kflag, s_abort, s_nev, st);
+            if (!step_end<float, Lat7, NT>(d, *reinterpret_cast<Scratch *>(s_in), st.t, it, it == nsteps - 1, st.G,
+                                           st.whole, st.budget, st.extra, &planned, gave_up))
+                break;
+            if (tid == 0) s_nev = 0;
+            if (tid < TMA_KFLAG_WORDS) kflag[tid] = 0u;
+            __syncthreads();
+        }
+        step_exit(d.sc, after);
+    }
 }
 
 // The kernel's shared-memory opt-in (once per device).
-template <bool NOISE>
+template <bool NOISE, bool FUSED = false>
 cudaError_t prepare_update7_tma()
 {
     static bool attr[64] = {};
@@ -468,7 +528,7 @@ cudaError_t prepare_update7_tma()
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !attr[dev]) {
-        e = cudaFuncSetAttribute(k_update7_tma<TMA7_TY, TMA7_STAGES, TMA7_CTAS, NOISE>,
+        e = cudaFuncSetAttribute(k_update7_tma<TMA7_TY, TMA7_STAGES, TMA7_CTAS, NOISE, FUSED>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)tma7_smem_bytes<TMA7_TY, TMA7_STAGES>());
         if (e != cudaSuccess) return e;
@@ -499,7 +559,36 @@ cudaError_t launch_update7_tma(const SimDev &d, const CUtensorMap *maps, bool pd
     la[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = la;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_update7_tma<TMA7_TY, TMA7_STAGES, TMA7_CTAS, NOISE>, d, maps[0], maps[1]);
+    return cudaLaunchKernelEx(&cfg, k_update7_tma<TMA7_TY, TMA7_STAGES, TMA7_CTAS, NOISE, false>, d, maps[0], maps[1],
+                              1);
+}
+
+// Many steps in one cooperative launch (with `maps` null, only whether it fits).
+template <bool NOISE>
+cudaError_t launch_steps7_tma(const SimDev &d, const CUtensorMap *maps, int steps, cudaStream_t s)
+{
+    cudaError_t e = prepare_update7_tma<NOISE, true>();
+    if (e != cudaSuccess) return e;
+    const auto kernel = k_update7_tma<TMA7_TY, TMA7_STAGES, TMA7_CTAS, NOISE, true>;
+    const size_t smem = tma7_smem_bytes<TMA7_TY, TMA7_STAGES>();
+    static int per_sm[64] = {};
+    if (!maps) return steps_fit((const void *)kernel, Tma7Geom<TMA7_TY>::NT, smem, d.upd_ctas, per_sm);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)d.upd_ctas);
+    cfg.blockDim = dim3(Tma7Geom<TMA7_TY>::NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute la[1];
+    la[0].id = cudaLaunchAttributeCooperative;
+    la[0].val.cooperative = 1;
+    cfg.attrs = la;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, d, maps[0], maps[1], steps);
+}
+
+inline cudaError_t launch_steps7_tma_any(const SimDev &d, const CUtensorMap *maps, int, int steps, cudaStream_t s)
+{
+    return d.noise_on ? launch_steps7_tma<true>(d, maps, steps, s) : launch_steps7_tma<false>(d, maps, steps, s);
 }
 
 inline cudaError_t launch_update7_tma_any(const SimDev &d, const CUtensorMap *maps, int, bool pdl, cudaStream_t s)

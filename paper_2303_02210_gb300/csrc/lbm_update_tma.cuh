@@ -1,6 +1,7 @@
 // TMA-staged fused update (FP32 or 16-bit storage, walls in y), the fast path
 // of App. A steps 1-7 (step 3's divisions are added to the staged tile): the
-// same per-node arithmetic as k_update, different data movement.
+// same per-node arithmetic as k_update, different data movement. One update a
+// launch, or many whole steps (FUSED, lbm_steps.cuh).
 //
 // Each CTA (persistent, CTAS per SM) walks tiles of 128 columns x TY rows of
 // the active window, dealt round-robin over the grid. A tile's pre-stream
@@ -34,6 +35,7 @@
 
 #include "lbm_kernels.cuh"
 #include "lbm_pair.cuh"
+#include "lbm_steps.cuh"
 #include "lbm_tma.cuh"
 
 namespace lbm {
@@ -83,7 +85,7 @@ constexpr size_t tma_smem_bytes()
 // on a 16-byte boundary.)
 template <typename S>
 struct TmaCfg {
-    static constexpr int TY0 = 2, CTAS0 = sizeof(S) == 4 ? 5 : 6, STAGES0 = sizeof(S) == 4 ? 2 : 2;
+    static constexpr int TY0 = 2, CTAS0 = sizeof(S) == 4 ? 5 : 6, STAGES0 = 2;
     static constexpr int TY1 = 4, CTAS1 = 3, STAGES1 = sizeof(S) == 4 ? 2 : 4;
     static constexpr int TY2 = 2, CTAS2 = 6, STAGES2 = 1;
 };
@@ -254,59 +256,32 @@ __device__ __forceinline__ float update_node(const float g[NQ], float rho, bool 
     return 0.0f;
 }
 
-// CTAS CTAs per SM (registers are capped so that they fit); NOISE: sigma != 0;
-// TSTORE: results leave through a shared output tile and one bulk tensor
-// store per tile (ts0 / ts1: copy 0 / 1 as [plane][row][stored column] with
-// the columns cut at x = W - 1, boxes of 128 x TY x 9), else per-lane stores.
-template <typename S, int TY, int STAGES, int CTAS, bool NOISE, bool TSTORE>
-__global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
-    k_update_tma(SimDev d, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
-                 const __grid_constant__ CUtensorMap ts0, const __grid_constant__ CUtensorMap ts1)
+// What one update leaves for the frame of a launch of many steps.
+struct TmaStep {
+    uint32_t t;       // the step
+    int tiles;        // tiles this CTA has staged since the launch began (stage and phase of the next)
+    int G, extra;     // planner CTAs of the step; arrivals waited for in vain (a failure-detection test)
+    bool whole;       // each planner CTA scans the whole front
+    long long budget; // of the bounded waits
+};
+
+// One update: the CTA's tiles of the step that the device scalars hold.
+// Returns whether a wait of this thread gave up.
+template <typename S, int TY, int STAGES, bool NOISE, bool TSTORE, bool FUSED>
+__device__ __forceinline__ bool update_tma_step(const SimDev &d, const CUtensorMap *tm0, const CUtensorMap *tm1,
+                                                const CUtensorMap *ts0, const CUtensorMap *ts1, S *s_in, S *s_out,
+                                                uint64_t *full, uint64_t *empty, int *ev_k, unsigned *kflag,
+                                                int &s_abort, int &s_nev, TmaStep &st)
 {
-    static_assert(!TSTORE || sizeof(S) == 4, "bulk tensor stores of 16-bit tiles would start off a 16-byte boundary");
     using G = TmaGeom<S, TY>;
     constexpr int NT = G::NT, PLANE = G::PLANE;
     const Pop<S> pc(d);
-    extern __shared__ __align__(128) float smem_f[];
-    // stages on a 128-byte boundary (offset from the array itself, so that
-    // every access stays a shared-memory access)
-    S *s_in = reinterpret_cast<S *>(smem_f + ((128u - (smem_u32(smem_f) & 127u)) & 127u) / 4u);
-    S *s_out = s_in + STAGES * G::STRIDE; // the output tile (TSTORE), on a 128-byte boundary
-    uint64_t *full = reinterpret_cast<uint64_t *>(s_out + (TSTORE ? 9 * TY * TMA_TX : 0));
-    uint64_t *empty = full + STAGES;
-    // divisions of this CTA's tiles: local tile index, two staged offsets, amount
-    int *ev_k = reinterpret_cast<int *>(empty + STAGES);
     int *ev_off = ev_k + TMA_EV_CAP;
     float *ev_add = reinterpret_cast<float *>(ev_off + 2 * TMA_EV_CAP);
-    unsigned *kflag = reinterpret_cast<unsigned *>(ev_add + TMA_EV_CAP); // tiles with divisions
-    __shared__ int s_abort, s_nev;
-
     const int W = d.W, H = d.H, Wp = d.Wp;
     const long long P = d.P;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int half = warp & 1, row = warp >> 1; // column half and row of the tile
-
-    // prologue, which may overlap the end of the planner (programmatic
-    // dependent launch): barriers, tensor map, tile flags
-    if (tid == 0) {
-        s_abort = 0;
-        s_nev = 0;
-        prefetch_tensormap(&tm0);
-        prefetch_tensormap(&tm1);
-        if (TSTORE) {
-            prefetch_tensormap(&ts0);
-            prefetch_tensormap(&ts1);
-        }
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], G::WARPS);
-        }
-        fence_mbar_init();
-    }
-    if (tid < TMA_KFLAG_WORDS) kflag[tid] = 0u;
-    __syncthreads();
-    // everything below reads what the planner wrote
-    grid_dependency_wait();
     // step t (read from the device, so a captured step replays as is) pulls
     // from copy t & 1 (tensor map tm0 or tm1) and writes the other
     const uint32_t t = (uint32_t)d.sc->step;
@@ -314,11 +289,17 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
     // withhold the bulk copies, so that the first wait of every thread runs out)
     const long long budget = d.sc->wait_budget > 0 ? d.sc->wait_budget : kWaitBudget;
     const bool withhold = (d.sc->wait_test & WAIT_TEST_COPIES) != 0;
+    st.t = t;
+    st.budget = budget;
+    if (FUSED) {
+        st.extra = (d.sc->wait_test & WAIT_TEST_BARRIER) ? 1 : 0;
+        st.G = step_planners<NT>(d.sc->plan_kc, d.MW, (int)gridDim.x, &st.whole);
+    }
     const int cur = (int)(t & 1u);
-    const CUtensorMap *tm = cur ? &tm1 : &tm0;
-    const CUtensorMap *ts = cur ? &ts0 : &ts1; // (the copy this step writes)
-    const S *__restrict__ fin = (const S *)d.f[cur];
-    S *__restrict__ fout = (S *)d.f[cur ^ 1];
+    const CUtensorMap *tm = cur ? tm1 : tm0;
+    const CUtensorMap *ts = cur ? ts0 : ts1; // (the copy this step writes)
+    const S *fin = (const S *)d.f[cur];
+    S *fout = (S *)d.f[cur ^ 1];
     const int y_r = d.sc->y_r, y_copy = d.sc->y_copy, y_hi = d.sc->y_hi;
 
     // rows the rear wall has just frozen: bring this copy up to date (whole
@@ -337,13 +318,14 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
     const int nty = nrows > 0 ? (nrows + TY - 1) / TY : 0;
     const int ntiles = ncx * nty;
     const int Gd = (int)gridDim.x;
+    const int base = st.tiles; // tiles this CTA has staged in the launch's steps before
     const int count = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / Gd + 1 : 0;
     // tile k of this CTA is blockIdx.x + k Gd; its (tx, ty) advance by (Gd % ncx, Gd / ncx)
     const int dtx = Gd % ncx, dty = Gd / ncx;
     // producer state (thread 0): next tile to load and copies issued
     int itx = (int)blockIdx.x % ncx, ity = (int)blockIdx.x / ncx, issued = 0;
     auto issue = [&]() {
-        const int s = issued % STAGES;
+        const int s = (base + issued) % STAGES;
         mbar_arrive_expect_tx(&full[s], G::BYTES);
         tma_load_3d(s_in + s * G::STRIDE, tm, itx * TMA_TX - 4 + kXO, y_r + ity * TY - 1, 0, &full[s]);
         ++issued;
@@ -370,15 +352,18 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
     auto amount = [&](int e) {
         return (float)((double)d.ev_count[(size_t)(t & 1u) * (size_t)d.ns_max + (size_t)e] * d.half_cell);
     };
-    const int mine = nev_all > 0 ? d.bucket_cnt[blockIdx.x] : 0;
-    if (mine <= TMA_EV_CAP) { // (the bucket holds kBucketCap >= TMA_EV_CAP records)
-        for (int j = tid; j < mine; j += NT) {
-            const int e = d.bucket[blockIdx.x * kBucketCap + j];
-            const int k = d.rec_k[e];
-            ev_k[j] = k;
-            ev_off[2 * j] = d.rec_off[2 * e];
-            ev_off[2 * j + 1] = d.rec_off[2 * e + 1];
-            ev_add[j] = amount(e);
+    // (one entry per thread, read without waiting for their number)
+    static_assert(NT >= TMA_EV_CAP && kBucketCap >= TMA_EV_CAP, "one bucket entry per thread");
+    const unsigned long long rec = d.inject_in_update && tid < TMA_EV_CAP ? d.bucket[blockIdx.x * kBucketCap + tid] : 0ull;
+    const int in_bucket = d.inject_in_update ? d.bucket_cnt[blockIdx.x] : 0;
+    const int mine = nev_all > 0 ? in_bucket : 0;
+    if (mine <= TMA_EV_CAP) {
+        if (tid < mine) {
+            const int k = rec_tile(rec);
+            ev_k[tid] = k;
+            ev_off[2 * tid] = rec_off0(rec);
+            ev_off[2 * tid + 1] = rec_off1(rec);
+            ev_add[tid] = amount(rec_rank(rec));
             if (k < 32 * TMA_KFLAG_WORDS) atomicOr(&kflag[k >> 5], 1u << (k & 31));
         }
         if (tid == 0) s_nev = mine;
@@ -396,11 +381,12 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
                 const int e = eb + j * NT + tid;
                 if (own[j] == (int)blockIdx.x) {
                     const int at = atomicAdd(&s_nev, 1);
-                    const int k = d.rec_k[e];
+                    const unsigned long long r = d.rec[e];
+                    const int k = rec_tile(r);
                     if (at < TMA_EV_CAP) {
                         ev_k[at] = k;
-                        ev_off[2 * at] = d.rec_off[2 * e];
-                        ev_off[2 * at + 1] = d.rec_off[2 * e + 1];
+                        ev_off[2 * at] = rec_off0(r);
+                        ev_off[2 * at + 1] = rec_off1(r);
                         ev_add[at] = amount(e);
                     }
                     if (k < 32 * TMA_KFLAG_WORDS) atomicOr(&kflag[k >> 5], 1u << (k & 31));
@@ -409,6 +395,19 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
         }
     }
     __syncthreads();
+    if (FUSED) {
+        // this CTA's bucket, its share of the merge table's entries and of the
+        // counts of the selection before the present one are emptied for the
+        // selection that follows this update
+        if (tid == 0 && d.inject_in_update) d.bucket_cnt[blockIdx.x] = 0;
+        const int nsel = d.sc->rec_n, nev = d.sc->n_events;
+        const size_t obuf = (size_t)((t + 1u) & 1u) * (size_t)d.ns_max;
+        for (int r = (int)blockIdx.x * NT + tid; r < nev; r += Gd * NT) d.ev_count[obuf + r] = 0;
+        for (int r = (int)blockIdx.x * NT + tid; r < nsel; r += Gd * NT) {
+            const int slot = d.hlist[r];
+            if (slot >= 0) d.htab[slot] = EMPTY_ENTRY;
+        }
+    }
     const int nev = s_nev;                     // divisions of this CTA
     const bool ev_overflow = nev > TMA_EV_CAP; // then scan the global list per tile
 
@@ -423,8 +422,8 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
     int tx = (int)blockIdx.x % ncx, ty = (int)blockIdx.x / ncx;
 
     for (int k = 0; k < count; ++k) {
-        const int s = k % STAGES;
-        const uint32_t parity = (uint32_t)((k / STAGES) & 1);
+        const int s = (base + k) % STAGES;
+        const uint32_t parity = (uint32_t)(((base + k) / STAGES) & 1);
         const int x0 = tx * TMA_TX, y0 = y_r + ty * TY;
         S *stage = s_in + s * G::STRIDE;
         if (!dead && !mbar_wait_bounded(&full[s], parity, budget)) {
@@ -441,16 +440,16 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
             };
             if (!ev_overflow) {
                 for (int i = tid; i < nev; i += NT)
-                    if (ev_k[i] == k) {
+                    if (ev_k[i] == k && ev_add[i] != 0.0f) { // (0: a repeat)
                         add_slot(ev_off[2 * i], ev_add[i]);
                         add_slot(ev_off[2 * i + 1], ev_add[i]);
                     }
             } else {
                 for (int e = tid; e < nev_all; e += NT)
-                    if (d.rec_owner[e] == (int)blockIdx.x && d.rec_k[e] == k) {
+                    if (d.rec_owner[e] == (int)blockIdx.x && rec_tile(d.rec[e]) == k) {
                         const float a = amount(e);
-                        add_slot(d.rec_off[2 * e], a);
-                        add_slot(d.rec_off[2 * e + 1], a);
+                        add_slot(rec_off0(d.rec[e]), a);
+                        add_slot(rec_off1(d.rec[e]), a);
                     }
             }
             fence_proxy_async_smem(); // before a later bulk copy overwrites them
@@ -635,20 +634,92 @@ __global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
         atomicOr(&d.sc->status, ST_TIMEOUT);
         // let the copies still in flight land before the CTA exits
         for (int k = issued - STAGES > 0 ? issued - STAGES : 0; k < issued; ++k)
-            mbar_wait_bounded(&full[k % STAGES], (uint32_t)((k / STAGES) & 1), kWaitBudget);
+            mbar_wait_bounded(&full[(base + k) % STAGES], (uint32_t)(((base + k) / STAGES) & 1), kWaitBudget);
     }
-    mass = warp_sum_ll(mass);
-    maxrow = warp_max_i(maxrow);
-    const double clipd = warp_sum_d((double)clip);
+    mass = warp_sum_u63(mass);
+    maxrow = __reduce_max_sync(0xffffffffu, maxrow);
+    const double clipd = __any_sync(0xffffffffu, clip != 0.0f) ? warp_sum_d((double)clip) : 0.0;
     if (lane == 0) {
         if (mass != 0) atomicAdd(&d.sc->mass_accum, (unsigned long long)mass);
         if (maxrow >= 0) atomicMax(&d.sc->maxmass_accum, maxrow);
         if (clipd != 0.0) atomicAdd(&d.sc->clip_mass, clipd);
     }
+    st.tiles = base + count;
+    return dead;
+}
+
+// CTAS CTAs per SM (registers are capped so that they fit); NOISE: sigma != 0;
+// TSTORE: results leave through a shared output tile and one bulk tensor
+// store per tile (ts0 / ts1: copy 0 / 1 as [plane][row][stored column] with
+// the columns cut at x = W - 1, boxes of 128 x TY x 9), else per-lane stores.
+// FUSED: `nsteps` whole steps in this launch (lbm_steps.cuh), else one update.
+template <typename S, int TY, int STAGES, int CTAS, bool NOISE, bool TSTORE, bool FUSED>
+__global__ void __launch_bounds__(TmaGeom<S, TY>::NT, CTAS)
+    k_update_tma(SimDev d, const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
+                 const __grid_constant__ CUtensorMap ts0, const __grid_constant__ CUtensorMap ts1, int nsteps)
+{
+    static_assert(!TSTORE || sizeof(S) == 4, "bulk tensor stores of 16-bit tiles would start off a 16-byte boundary");
+    using G = TmaGeom<S, TY>;
+    extern __shared__ __align__(128) float smem_f[];
+    // stages on a 128-byte boundary (offset from the array itself, so that
+    // every access stays a shared-memory access)
+    S *s_in = reinterpret_cast<S *>(smem_f + ((128u - (smem_u32(smem_f) & 127u)) & 127u) / 4u);
+    S *s_out = s_in + STAGES * G::STRIDE; // the output tile (TSTORE), on a 128-byte boundary
+    uint64_t *full = reinterpret_cast<uint64_t *>(s_out + (TSTORE ? 9 * TY * TMA_TX : 0));
+    uint64_t *empty = full + STAGES;
+    // divisions of this CTA's tiles: local tile index, two staged offsets, amount
+    int *ev_k = reinterpret_cast<int *>(empty + STAGES);
+    unsigned *kflag = reinterpret_cast<unsigned *>(ev_k + 4 * TMA_EV_CAP); // tiles with divisions
+    __shared__ int s_abort, s_nev;
+    const int tid = threadIdx.x;
+
+    // prologue, which may overlap the end of the planner (programmatic
+    // dependent launch): barriers, tensor map, tile flags
+    if (tid == 0) {
+        s_abort = 0;
+        s_nev = 0;
+        prefetch_tensormap(&tm0);
+        prefetch_tensormap(&tm1);
+        if (TSTORE) {
+            prefetch_tensormap(&ts0);
+            prefetch_tensormap(&ts1);
+        }
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], G::WARPS);
+        }
+        fence_mbar_init();
+    }
+    if (tid < TMA_KFLAG_WORDS) kflag[tid] = 0u;
+    __syncthreads();
+    // everything below reads what the planner wrote
+    grid_dependency_wait();
+    TmaStep st;
+    st.tiles = 0;
+    if constexpr (!FUSED) {
+        update_tma_step<S, TY, STAGES, NOISE, TSTORE, false>(d, &tm0, &tm1, &ts0, &ts1, s_in, s_out, full, empty, ev_k,
+                                                             kflag, s_abort, s_nev, st);
+    } else {
+        using Scratch = StepScratch<G::NT>;
+        static_assert(sizeof(Scratch) <= (size_t)STAGES * G::STRIDE * sizeof(S), "the planner's room");
+        const long long after = d.sc->step + nsteps;
+        unsigned long long planned = 0;
+        for (int it = 0; it < nsteps; ++it) {
+            const bool gave_up = update_tma_step<S, TY, STAGES, NOISE, TSTORE, true>(
+                d, &tm0, &tm1, &ts0, &ts1, s_in, s_out, full, empty, ev_k, kflag, s_abort, s_nev, st);
+            if (!step_end<S, Lat9, G::NT>(d, *reinterpret_cast<Scratch *>(s_in), st.t, it, it == nsteps - 1, st.G,
+                                          st.whole, st.budget, st.extra, &planned, gave_up))
+                break;
+            if (tid == 0) s_nev = 0;
+            if (tid < TMA_KFLAG_WORDS) kflag[tid] = 0u;
+            __syncthreads();
+        }
+        step_exit(d.sc, after);
+    }
 }
 
 // The kernel's shared-memory opt-in (once per device).
-template <typename S, int TY, int STAGES, int CTAS, bool NOISE, bool TSTORE>
+template <typename S, int TY, int STAGES, int CTAS, bool NOISE, bool TSTORE, bool FUSED = false>
 cudaError_t prepare_update_tma_variant()
 {
     static bool attr[64] = {};
@@ -656,7 +727,7 @@ cudaError_t prepare_update_tma_variant()
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !attr[dev]) {
-        e = cudaFuncSetAttribute(k_update_tma<S, TY, STAGES, CTAS, NOISE, TSTORE>,
+        e = cudaFuncSetAttribute(k_update_tma<S, TY, STAGES, CTAS, NOISE, TSTORE, FUSED>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)tma_smem_bytes<S, TY, STAGES, TSTORE>());
         if (e != cudaSuccess) return e;
@@ -684,8 +755,49 @@ cudaError_t launch_update_tma_variant(const SimDev &d, const CUtensorMap *maps, 
     la[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = la;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_update_tma<S, TY, STAGES, CTAS, NOISE, TSTORE>, d, maps[0], maps[1],
-                              maps[TSTORE ? 2 : 0], maps[TSTORE ? 3 : 1]);
+    return cudaLaunchKernelEx(&cfg, k_update_tma<S, TY, STAGES, CTAS, NOISE, TSTORE, false>, d, maps[0], maps[1],
+                              maps[TSTORE ? 2 : 0], maps[TSTORE ? 3 : 1], 1);
+}
+
+// A cooperative launch: every CTA resident (they wait for one another). With
+// `maps` null, only whether it fits.
+template <typename S, int TY, int STAGES, int CTAS, bool NOISE, bool TSTORE>
+cudaError_t launch_steps_tma_variant(const SimDev &d, const CUtensorMap *maps, int steps, cudaStream_t s)
+{
+    cudaError_t e = prepare_update_tma_variant<S, TY, STAGES, CTAS, NOISE, TSTORE, true>();
+    if (e != cudaSuccess) return e;
+    const auto kernel = k_update_tma<S, TY, STAGES, CTAS, NOISE, TSTORE, true>;
+    const size_t smem = tma_smem_bytes<S, TY, STAGES, TSTORE>();
+    static int per_sm[64] = {};
+    if (!maps) return steps_fit((const void *)kernel, TmaGeom<S, TY>::NT, smem, d.upd_ctas, per_sm);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)d.upd_ctas);
+    cfg.blockDim = dim3(TmaGeom<S, TY>::NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute la[1];
+    la[0].id = cudaLaunchAttributeCooperative;
+    la[0].val.cooperative = 1;
+    cfg.attrs = la;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, d, maps[0], maps[1], maps[TSTORE ? 2 : 0], maps[TSTORE ? 3 : 1], steps);
+}
+
+template <typename S, bool NOISE>
+cudaError_t launch_steps_tma_noise(const SimDev &d, const CUtensorMap *maps, int variant, int steps, cudaStream_t s)
+{
+    using C = TmaCfg<S>;
+    if (variant == 1) return launch_steps_tma_variant<S, C::TY1, C::STAGES1, C::CTAS1, NOISE, false>(d, maps, steps, s);
+    if constexpr (sizeof(S) == 4)
+        if (variant == 2) return launch_steps_tma_variant<S, C::TY2, C::STAGES2, C::CTAS2, NOISE, true>(d, maps, steps, s);
+    return launch_steps_tma_variant<S, C::TY0, C::STAGES0, C::CTAS0, NOISE, false>(d, maps, steps, s);
+}
+
+template <typename S>
+cudaError_t launch_steps_tma(const SimDev &d, const CUtensorMap *maps, int variant, int steps, cudaStream_t s)
+{
+    return d.noise_on ? launch_steps_tma_noise<S, true>(d, maps, variant, steps, s)
+                      : launch_steps_tma_noise<S, false>(d, maps, variant, steps, s);
 }
 
 template <typename S, bool NOISE>
