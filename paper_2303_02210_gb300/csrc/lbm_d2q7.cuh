@@ -165,7 +165,15 @@ __device__ __forceinline__ void collide7(const R *g, R rho, R *fo, const Consts<
     R jx, jy;
     momentum7<R>(g, jx, jy);
     if constexpr (sizeof(R) == 8) {
-        const R ux = jx / rho, uy = jy / rho;
+        R ux, uy;
+        const SharedDiv<R> by_rho(rho);
+        if (by_rho.ok && SharedDiv<R>::fits(jx) && SharedDiv<R>::fits(jy)) {
+            ux = by_rho.quot(jx);
+            uy = by_rho.quot(jy);
+        } else {
+            ux = jx / rho;
+            uy = jy / rho;
+        }
         const R usx = c.cmu * ux, usy = c.cmu * uy; // u* = (1 - mu) u
         const R uu = usx * usx + usy * usy;
 #pragma unroll
@@ -211,13 +219,17 @@ __device__ __forceinline__ void noise_eta7(R *eta, const u32x4 &w, const Consts<
     uint32_t m[NQ7];
     noise_fields7(w, m);
     if constexpr (sizeof(R) == 8) {
+        // u_i = (2 m_i + 1) 2^-19 in the low bits of a double of magnitude 2^33;
+        // their sum, exact in any order, as an integer
         double u[NQ7];
+        uint32_t sum = 0;
 #pragma unroll
-        for (int i = 0; i < NQ7; ++i) u[i] = ((double)m[i] + 0.5) * 3.814697265625e-06;
-        double S = u[0];
-#pragma unroll
-        for (int i = 1; i < NQ7; ++i) S = S + u[i];
-        const double ubar = S / 7.0;
+        for (int i = 0; i < NQ7; ++i) {
+            u[i] = __hiloint2double(0x42000000, (int)(2u * m[i] + 1u)) - 8589934592.0;
+            sum += 2u * m[i] + 1u;
+        }
+        const double S = __hiloint2double(0x42000000, (int)sum) - 8589934592.0;
+        const double ubar = SharedDiv<double>(7.0, 1.0 / 7.0).quot(S);
 #pragma unroll
         for (int i = 0; i < NQ7; ++i) eta[i] = c.two_sigma * (u[i] - ubar);
     } else {
@@ -239,6 +251,13 @@ template <typename R>
 __device__ __forceinline__ R fix_negative7(R *fo, int mode)
 {
     R added = R(0);
+    if constexpr (sizeof(R) == 8) {
+        // no sign bit, no negative (a test on the integer pipe)
+        int any = 0;
+#pragma unroll
+        for (int i = 0; i < NQ7; ++i) any |= __double2hiint(fo[i]);
+        if (any >= 0) return added;
+    }
     R mn = fo[0];
 #pragma unroll
     for (int i = 1; i < NQ7; ++i) mn = mn < fo[i] ? mn : fo[i];
@@ -252,8 +271,7 @@ __device__ __forceinline__ R fix_negative7(R *fo, int mode)
             R sm = fo[0];
 #pragma unroll
             for (int i = 1; i < NQ7; ++i) sm = sm + fo[i];
-#pragma unroll
-            for (int i = 0; i < NQ7; ++i) fo[i] = (r0 * fo[i]) / sm;
+            scale_by_quotient<R, NQ7>(fo, r0, sm);
         }
 #pragma unroll
         for (int i = 1; i < NQ7; ++i)
@@ -273,8 +291,7 @@ __device__ __forceinline__ R fix_negative7(R *fo, int mode)
         R sm = fo[0];
 #pragma unroll
         for (int i = 1; i < NQ7; ++i) sm = sm + fo[i];
-#pragma unroll
-        for (int i = 0; i < NQ7; ++i) fo[i] = (r0 * fo[i]) / sm;
+        scale_by_quotient<R, NQ7>(fo, r0, sm);
     }
     return added;
 }

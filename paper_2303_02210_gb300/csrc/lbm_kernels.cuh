@@ -18,6 +18,7 @@
 #pragma once
 
 #include "lbm_common.cuh"
+#include "lbm_div.cuh"
 
 namespace lbm {
 
@@ -37,7 +38,14 @@ __device__ __forceinline__ long long fix24<float>(float r)
     return v < 8388608.0f ? lo : hi; // v < 2^63 always (rho < 2^39)
 }
 template <>
-__device__ __forceinline__ long long fix24<double>(double r) { return __double2ll_rn(r * 16777216.0); }
+__device__ __forceinline__ long long fix24<double>(double r)
+{
+    // r 2^24 rounded into the low bits of a double of magnitude 1.5 2^52 (to
+    // nearest, ties to even, as the conversion does): one FP64 operation
+    const double magic = 6755399441055744.0;
+    if ((__double2hiint(r) & 0x7FFFFFFF) >= 0x41900000) return __double2ll_rn(r * 16777216.0);
+    return __double_as_longlong(__fma_rn(r, 16777216.0, magic)) - __double_as_longlong(magic);
+}
 
 // Occupancy threshold in the storage type (the FP32 copy is rounded on the host).
 template <typename R>
@@ -376,17 +384,32 @@ __device__ __forceinline__ void collide(const R *g, R rho, R *fo, const Consts<R
     const R jx = ((((g[1] - g[3]) + g[5]) - g[6]) - g[7]) + g[8];
     const R jy = ((((g[2] - g[4]) + g[5]) + g[6]) - g[7]) - g[8];
     if constexpr (sizeof(R) == 8) {
-        const R ux = jx / rho, uy = jy / rho;
+        R ux, uy;
+        const SharedDiv<R> by_rho(rho);
+        if (by_rho.ok && SharedDiv<R>::fits(jx) && SharedDiv<R>::fits(jy)) {
+            ux = by_rho.quot(jx);
+            uy = by_rho.quot(jy);
+        } else {
+            ux = jx / rho;
+            uy = jy / rho;
+        }
         const R usx = c.cmu * ux, usy = c.cmu * uy; // u* = (1 - mu) u
         const R uu = usx * usx + usy * usy;
-        const R eu[NQ] = {R(0), usx, usy, -usx, -usy, usx + usy, -usx + usy, -usx - usy, usx - usy};
+        // opposite directions share 4.5 (e.u)^2 and differ in the sign of 3 e.u
+        // (a negation is exact, so each value is that of its own formula)
+        const R m = R(1.5) * uu;
+        auto relax = [&](int i, R t1) {
+            const R fss = (wq<R>(i) * rho) * (t1 - m);  // Eq. 3, D2Q9
+            fo[i] = g[i] - c.omega * (g[i] - fss);     // Eq. 2
+        };
+        relax(0, R(1));
 #pragma unroll
-        for (int i = 0; i < NQ; ++i) {
-            R t1 = R(1) + R(3) * eu[i];
-            t1 = t1 + R(4.5) * (eu[i] * eu[i]);
-            t1 = t1 - R(1.5) * uu;
-            const R fss = (wq<R>(i) * rho) * t1;    // Eq. 3, D2Q9
-            fo[i] = g[i] - c.omega * (g[i] - fss); // Eq. 2
+        for (int k = 0; k < 4; ++k) {
+            const int i = k == 0 ? 1 : (k == 1 ? 2 : (k == 2 ? 5 : 6));
+            const R eu = i == 1 ? usx : (i == 2 ? usy : (i == 5 ? usx + usy : -usx + usy));
+            const R s3 = R(3) * eu, sq = R(4.5) * (eu * eu);
+            relax(i, (R(1) + s3) + sq);
+            relax(opp(i), (R(1) - s3) + sq);
         }
         if (eta) {
 #pragma unroll
@@ -452,13 +475,17 @@ __device__ __forceinline__ void noise_eta_words(R *eta, const u32x4 &w, const Co
     uint32_t m[NQ];
     noise_fields(w, m);
     if constexpr (sizeof(R) == 8) {
+        // u_i = (2 m_i + 1) 2^-15 in the low bits of a double of magnitude 2^37;
+        // their sum, exact in any order, as an integer
         double u[NQ];
+        uint32_t sum = 0;
 #pragma unroll
-        for (int i = 0; i < NQ; ++i) u[i] = ((double)m[i] + 0.5) * 6.103515625e-05;
-        double S = u[0];
-#pragma unroll
-        for (int i = 1; i < NQ; ++i) S = S + u[i];
-        const double ubar = S / 9.0;
+        for (int i = 0; i < NQ; ++i) {
+            u[i] = __hiloint2double(0x42400000, (int)(2u * m[i] + 1u)) - 137438953472.0;
+            sum += 2u * m[i] + 1u;
+        }
+        const double S = __hiloint2double(0x42400000, (int)sum) - 137438953472.0;
+        const double ubar = SharedDiv<double>(9.0, 1.0 / 9.0).quot(S);
 #pragma unroll
         for (int i = 0; i < NQ; ++i) eta[i] = c.two_sigma * (u[i] - ubar);
     } else {
@@ -564,6 +591,12 @@ __device__ __forceinline__ R fix_negative(R *fo, int mode)
         const float mn = fminf(fminf(fminf(fo[0], fo[1]), fminf(fo[2], fo[3])),
                                fminf(fminf(fo[4], fo[5]), fminf(fminf(fo[6], fo[7]), fo[8])));
         if (mn >= 0.0f) return added; // the common case
+    } else {
+        // no sign bit, no negative (a test on the integer pipe)
+        int any = 0;
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) any |= __double2hiint(fo[i]);
+        if (any >= 0) return added;
     }
     if (mode == 0) {
         if (fo[0] < R(0)) {
@@ -574,8 +607,7 @@ __device__ __forceinline__ R fix_negative(R *fo, int mode)
             R sm = fo[0];
 #pragma unroll
             for (int i = 1; i < NQ; ++i) sm = sm + fo[i];
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) fo[i] = (r0 * fo[i]) / sm;
+            scale_by_quotient<R, NQ>(fo, r0, sm);
         }
 #pragma unroll
         for (int i = 1; i < NQ; ++i) {
@@ -599,8 +631,7 @@ __device__ __forceinline__ R fix_negative(R *fo, int mode)
             R sm = fo[0];
 #pragma unroll
             for (int i = 1; i < NQ; ++i) sm = sm + fo[i];
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) fo[i] = (r0 * fo[i]) / sm;
+            scale_by_quotient<R, NQ>(fo, r0, sm);
         }
     }
     return added;
