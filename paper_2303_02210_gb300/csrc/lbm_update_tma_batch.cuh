@@ -182,9 +182,10 @@ __global__ void __launch_bounds__(TmaGeom<S, 2>::NT, CTAS)
     // the batch's tiles dealt in chunks of C consecutive tiles: chunk j to
     // CTA j mod G (a CTA's tiles then change member, which costs a tensor-map
     // fence and an accumulator flush, C times less often). kTmaBatchChunk, or
-    // less while a CTA has fewer than four chunks: the last round of chunks
-    // leaves CTAs idle (the 256-member ensemble 517 -> 506 us per step)
-    const int cs = T >= 4 * kTmaBatchChunk * Gd ? 3 : (T >= 16 * Gd ? 2 : (T >= 8 * Gd ? 1 : 0));
+    // just enough for one chunk per CTA when there are fewer tiles (chunks of
+    // 8 then leave most CTAs without one: a step of two served FP16
+    // members 62.0 -> 54.0 us)
+    const int cs = T > 4 * Gd ? 3 : (T > 2 * Gd ? 2 : (T > Gd ? 1 : 0));
     static_assert(kTmaBatchChunk == 8, "cs: log2 of the chunk");
     const int C = 1 << cs;
     const int nchunks = (T + C - 1) >> cs;
