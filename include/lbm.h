@@ -175,7 +175,8 @@ int lbm_create(const lbm_params_t *params, void *stream, void *arena, uint64_t a
 /* Advances `nsteps` time steps (App. A steps 1-7 each, plus the front
  * heights, Eq. 6 width, rear wall and active mass), all on the device with no
  * host synchronisation. With update_kernel 0 and an initial active window up to
- * a few million nodes (D2Q7: any), up to 64 steps are one cooperative launch;
+ * a few million nodes (D2Q7: any), up to 64 steps are one cooperative launch (a
+ * call of a single step only for small windows);
  * otherwise, and in kernel timing, a step is an update and a planner launch.
  * The results are the same bit for bit. Returns LBM_OK or a launch error; device-side status
  * (LBM_STATUS_*) is reported by lbm_stats. */

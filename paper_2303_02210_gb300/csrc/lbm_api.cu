@@ -229,17 +229,9 @@ void front_rows(const lbm_params_t &p, std::vector<int32_t> &rows)
     }
 }
 
-// Whether steps run many to a launch (lbm_steps.cuh) rather than as two
-// launches each: while the step's fixed cost counts. By the nodes of the
-// initial active window (rows0: its front), us per step in one launch
-// against two launches: FP32 27 against 33 or less at 0.5M nodes, 44 / 47 at
-// 2.1M, 70.0 / 71.5 at 4.2M, 118.6 / 117.2 at 8.4M (a lone update then has
-// fewer spills and the planner's share is small); 16 bits, which are bound by
-// their instructions, 43.4 / 45.7 at 2.1M, 73.2 / 72.3 at 4.2M, 118.4 /
-// 114.0 at 8.4M; D2Q7 105.6 / 109.6 at 8.4M still.
-bool fused_pays(const lbm_params_t &p, const std::vector<int32_t> &rows0)
+// Nodes of the initial active window (rows0: its front).
+long long window_nodes(const lbm_params_t &p, const std::vector<int32_t> &rows0)
 {
-    if (p.lattice == LBM_D2Q7) return true;
     long long top = 0, sum = 0;
     for (int32_t r : rows0) {
         top = std::max<long long>(top, r);
@@ -248,9 +240,24 @@ bool fused_pays(const lbm_params_t &p, const std::vector<int32_t> &rows0)
     long long rear = 0;
     if (p.wall_mode == LBM_WALL_ADVANCE)
         rear = (long long)std::max(0.0, std::floor((double)sum / p.width - p.wall_min_gap));
-    const long long nodes = (std::min<long long>(p.height, top + 2) - rear) * p.width;
-    return nodes <= (p.precision == LBM_FP32 ? 6ll << 20 : 4ll << 20);
+    return (std::min<long long>(p.height, top + 2) - rear) * p.width;
 }
+
+// Whether steps run many to a launch (lbm_steps.cuh) rather than as two
+// launches each: while the step's fixed cost counts. By the window's nodes, us
+// per step in one launch against two: FP32 23 against 27 at 0.5M nodes, 44 / 47
+// at 2.1M, 70.0 / 71.5 at 4.2M (as long over 20 steps, with the launch),
+// 118.6 / 117.2 at 8.4M (a lone update then has fewer spills and the planner's
+// share is small); 16 bits, which are bound by their instructions, 43.4 / 45.7
+// at 2.1M, 73.2 / 72.3 at 4.2M, 118.4 / 114.0 at 8.4M; D2Q7 63.5 / 65.2 at 4.2M,
+// 105.6 / 109.6 at 8.4M.
+bool fused_pays(const lbm_params_t &p, long long nodes) { return p.lattice == LBM_D2Q7 || nodes <= 3ll << 20; }
+
+// Whether a call of a single step takes the two launches all the same: they
+// overlap with the launches around them (programmatic dependents), which a
+// cooperative launch does not. Single steps of 2048 x 512 nodes 33.6 us against
+// 35.2, of 1024 x 256 24.3 against 25.2, of 512 x 52 21.3 against 19.3.
+bool lone_step_splits(const lbm_params_t &p, long long nodes) { return p.lattice == LBM_D2Q9 && nodes >= 1ll << 19; }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no
 // link-time dependency on the driver library).
@@ -309,7 +316,8 @@ struct lbm_sim {
     int64_t launches;
     // TMA-staged update (FP32, walls in y)
     bool use_tma;
-    bool fused; // many steps in one launch (update_kernel 0)
+    bool fused;       // many steps in one launch (update_kernel 0),
+    bool lone_splits; // but a call of one step as two launches
     int tma_grid, tma_variant;
     CUtensorMap maps[4]; // loads from copy 0, 1; stores into copy 0, 1 (variants that store in bulk)
     // kernel timing
@@ -631,6 +639,8 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
     }
     std::vector<int32_t> rows;
     front_rows(*p, rows);
+    const long long nodes = window_nodes(*p, rows);
+    s->lone_splits = lone_step_splits(*p, nodes);
     s->use_tma = s->fused = false;
     s->tma_grid = nsm;
     // staged update variant (KernelTable::tma_info): "tma" 0 (two-row tiles),
@@ -691,7 +701,7 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
             s->use_tma = false;
             d.inject_in_update = 0;
         }
-        s->fused = s->use_tma && p->update_kernel == 0 && s->kt->tma_steps && fused_pays(*p, rows) &&
+        s->fused = s->use_tma && p->update_kernel == 0 && s->kt->tma_steps && fused_pays(*p, nodes) &&
                    s->kt->tma_steps(d, nullptr, variant, 0, s->stream) == cudaSuccess;
         if (!ok && p->update_kernel >= 2 && p->update_kernel != 5) {
             if (s->own_arena) cudaFree(s->arena);
@@ -702,7 +712,8 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
 
     int rc = LBM_OK;
     do {
-        cudaError_t e = cudaMemsetAsync(s->arena, 0, L.total, s->stream);
+        // (the population copies, most of the arena, are all written by fill)
+        cudaError_t e = cudaMemsetAsync(base + L.off_mask, 0, L.total - L.off_mask, s->stream);
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         // the division table starts empty (every entry all ones)
         e = cudaMemsetAsync(d.htab, 0xFF, (size_t)L.hcap * 8u, s->stream);
@@ -729,10 +740,10 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
 static cudaError_t launch_update(lbm_sim *s, cudaStream_t st, bool pdl = true)
 {
     if (!s->d.inject_in_update && s->p.growth_mode != LBM_GROW_NONE) {
-        cudaError_t e = s->kt->inject(s->d, st);
+        cudaError_t e = s->kt->inject(s->d, pdl, st);
         if (e != cudaSuccess) return e;
     }
-    return s->use_tma ? s->kt->tma_update(s->d, s->maps, s->tma_variant, pdl, st) : s->kt->update(s->d, st);
+    return s->use_tma ? s->kt->tma_update(s->d, s->maps, s->tma_variant, pdl, st) : s->kt->update(s->d, pdl, st);
 }
 
 // Host-side mirror of one completed step (the kernels keep theirs on the device).
@@ -747,7 +758,7 @@ int lbm_step(lbm_sim *s, int64_t nsteps)
 {
     if (!s || nsteps < 0) return LBM_ERR_INVALID_ARG;
     USE_DEVICE(s);
-    if (s->fused && !s->timing) {
+    if (s->fused && !s->timing && !(nsteps == 1 && s->lone_splits)) {
         // (launches of at most kStepsPerLaunch steps: work on other streams
         // gets its turn between them)
         for (int64_t left = nsteps; left > 0;) {

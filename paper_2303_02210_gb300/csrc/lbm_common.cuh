@@ -252,8 +252,9 @@ struct KernelTable {
     // current state) and select the divisions of the next step
     cudaError_t (*plan)(const SimDev &, int init, cudaStream_t);
     // the selected divisions of the coming step (update kernels without staging)
-    cudaError_t (*inject)(const SimDev &, cudaStream_t);
-    cudaError_t (*update)(const SimDev &, cudaStream_t);
+    // (pdl: as a programmatic dependent of the kernel before it)
+    cudaError_t (*inject)(const SimDev &, bool pdl, cudaStream_t);
+    cudaError_t (*update)(const SimDev &, bool pdl, cudaStream_t);
     cudaError_t (*fields)(const SimDev &, int cur, double *rho, double *ux, double *uy, cudaStream_t);
     int (*plan_blocks_per_sm)(int batch); // of the own planner (0) or the batched one (1)
     int (*update_blocks_per_sm)();

@@ -484,6 +484,7 @@ __device__ __forceinline__ void update7_body(const SimDev &d, int blk, int nblk)
 template <typename S, int TPB, int NR>
 __global__ void __launch_bounds__(TPB) k_update7(SimDev d)
 {
+    grid_dependency_wait(); // the injected divisions
     update7_body<S, TPB, NR>(d, (int)blockIdx.x, (int)gridDim.x);
 }
 

@@ -34,15 +34,13 @@ struct Launch {
     {
         return launch_plan<S>(d, init, s);
     }
-    static cudaError_t inject(const SimDev &d, cudaStream_t s)
+    static cudaError_t inject(const SimDev &d, bool pdl, cudaStream_t s)
     {
-        k_inject<S><<<152, 128, 0, s>>>(d);
-        return cudaGetLastError();
+        return launch_dependent(k_inject<S, Lat9>, 152, 128, 0, pdl, s, d);
     }
-    static cudaError_t update(const SimDev &d, cudaStream_t s)
+    static cudaError_t update(const SimDev &d, bool pdl, cudaStream_t s)
     {
-        k_update<S, UPD_TPB, UPD_NR><<<d.update_grid, UPD_TPB, 0, s>>>(d);
-        return cudaGetLastError();
+        return launch_dependent(k_update<S, UPD_TPB, UPD_NR>, d.update_grid, UPD_TPB, 0, pdl, s, d);
     }
     static cudaError_t fields(const SimDev &d, int cur, double *rho, double *ux, double *uy, cudaStream_t s)
     {
@@ -50,13 +48,11 @@ struct Launch {
     }
     static cudaError_t batch_inject(const SimDev *ds, int nslots, int grid, cudaStream_t s)
     {
-        k_inject_batch<S><<<grid, INJ_NT, 0, s>>>(ds, nslots);
-        return cudaGetLastError();
+        return launch_dependent(k_inject_batch<S, Lat9>, grid, INJ_NT, 0, false, s, ds, nslots);
     }
     static cudaError_t batch_update(const SimDev *ds, const int4 *bm, int nb, cudaStream_t s)
     {
-        k_update_batch<S, UPD_TPB, UPD_NR><<<nb, UPD_TPB, 0, s>>>(ds, bm);
-        return cudaGetLastError();
+        return launch_dependent(k_update_batch<S, UPD_TPB, UPD_NR>, nb, UPD_TPB, 0, false, s, ds, bm);
     }
     static cudaError_t batch_plan(const SimDev *ds, int nslots, int cap, cudaStream_t s)
     {
@@ -118,15 +114,13 @@ struct Launch7 {
     {
         return launch_plan<S, Lat7>(d, init, s);
     }
-    static cudaError_t inject(const SimDev &d, cudaStream_t s)
+    static cudaError_t inject(const SimDev &d, bool pdl, cudaStream_t s)
     {
-        k_inject<S, Lat7><<<152, 128, 0, s>>>(d);
-        return cudaGetLastError();
+        return launch_dependent(k_inject<S, Lat7>, 152, 128, 0, pdl, s, d);
     }
-    static cudaError_t update(const SimDev &d, cudaStream_t s)
+    static cudaError_t update(const SimDev &d, bool pdl, cudaStream_t s)
     {
-        k_update7<S, UPD_TPB, UPD_NR><<<d.update_grid, UPD_TPB, 0, s>>>(d);
-        return cudaGetLastError();
+        return launch_dependent(k_update7<S, UPD_TPB, UPD_NR>, d.update_grid, UPD_TPB, 0, pdl, s, d);
     }
     static cudaError_t fields(const SimDev &d, int cur, double *rho, double *ux, double *uy, cudaStream_t s)
     {
@@ -134,13 +128,11 @@ struct Launch7 {
     }
     static cudaError_t batch_inject(const SimDev *ds, int nslots, int grid, cudaStream_t s)
     {
-        k_inject_batch<S, Lat7><<<grid, INJ_NT, 0, s>>>(ds, nslots);
-        return cudaGetLastError();
+        return launch_dependent(k_inject_batch<S, Lat7>, grid, INJ_NT, 0, false, s, ds, nslots);
     }
     static cudaError_t batch_update(const SimDev *ds, const int4 *bm, int nb, cudaStream_t s)
     {
-        k_update7_batch<S, UPD_TPB, UPD_NR><<<nb, UPD_TPB, 0, s>>>(ds, bm);
-        return cudaGetLastError();
+        return launch_dependent(k_update7_batch<S, UPD_TPB, UPD_NR>, nb, UPD_TPB, 0, false, s, ds, bm);
     }
     static cudaError_t batch_plan(const SimDev *ds, int nslots, int cap, cudaStream_t s)
     {

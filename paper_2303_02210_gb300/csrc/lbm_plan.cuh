@@ -119,11 +119,13 @@ __device__ __forceinline__ int plan_block_exscan(int v, int *total, int *s_i)
 // pair) and counted at the rank of the pair's first draw (ev_count of a
 // repeat stays 0; the counts were zero before this selection). The rank's list
 // entry is the table slot if this draw was the first of its (node, pair),
-// else -1. For the TMA-staged update, every draw also gets its record and a
-// place in its owner CTA's bucket (y_r: the rear wall of the coming step),
-// a repeat too (its amount is then 0 and the update skips it): the bucket's
-// atomic does not wait for the table's.
-template <typename R, typename LT = Lat9>
+// else -1. For the TMA-staged update, a first draw also gets its record and a
+// place in its owner CTA's bucket (y_r: the rear wall of the coming step).
+// EARLY: every draw does, a repeat too (its amount is then 0 and the update
+// skips it), so that the bucket's atomic does not wait for the table's: a
+// shorter chain, but one more atomic in flight and more registers (the batched
+// planners are 1% faster without).
+template <typename R, bool EARLY, typename LT = Lat9>
 __device__ __forceinline__ void plan_select(const SimDev &d, uint32_t key, int rank, size_t buf, int y_r)
 {
     EventTable tb;
@@ -136,7 +138,7 @@ __device__ __forceinline__ void plan_select(const SimDev &d, uint32_t key, int r
             owner = division_record<R>(d, rank, key, y_r, &rec);
         else
             owner = division_record7(d, rank, key, y_r, &rec);
-        at = atomicAdd(&d.bucket_cnt[owner], 1);
+        if (EARLY) at = atomicAdd(&d.bucket_cnt[owner], 1);
     }
     int first;
     const int slot = table_insert(tb, key, rank, &first);
@@ -144,6 +146,7 @@ __device__ __forceinline__ void plan_select(const SimDev &d, uint32_t key, int r
     d.ev_key[buf + rank] = key;
     if (first >= 0) atomicAdd(&d.ev_count[buf + first], 1);
     if (d.inject_in_update) {
+        if (!EARLY && slot >= 0) at = atomicAdd(&d.bucket_cnt[owner], 1);
         if (at < kBucketCap) d.bucket[(size_t)owner * kBucketCap + at] = rec;
         d.rec[rank] = rec;
         d.rec_owner[rank] = slot >= 0 ? owner : -1;
@@ -519,7 +522,7 @@ __device__ __forceinline__ void plan_body(const SimDev &d, int init, int G, int 
             if (lr >= 0) {
                 const long long rank = before + lr;
                 if (rank == ns - 1) s_kstop = (unsigned long long)(blk * C + j + 1);
-                if (rank < ns) plan_select<R, LT>(d, s_key[j], (int)rank, buf, nyr);
+                if (rank < ns) plan_select<R, false, LT>(d, s_key[j], (int)rank, buf, nyr);
             }
         }
         acc = total;
@@ -568,7 +571,7 @@ __device__ __forceinline__ void plan_body(const SimDev &d, int init, int G, int 
                 if (lr < 0) continue;
                 const long long rank = acc + bf + pr + lr;
                 if (rank == ns - 1) s_kstop = (unsigned long long)(k0 + i + 1);
-                if (rank < ns) plan_select<R, LT>(d, s_key[tid * PLAN_R + i], (int)rank, buf, nyr);
+                if (rank < ns) plan_select<R, false, LT>(d, s_key[tid * PLAN_R + i], (int)rank, buf, nyr);
             }
             acc += tt;
             base += (long long)G * PLAN_NT * PLAN_R;
@@ -669,7 +672,7 @@ __global__ void __launch_bounds__(PLAN_NT) k_plan(SimDev d, int init)
 // while the planners run) + the lattice width (the front scans) + a fixed
 // floor (the barriers and the commit). With tau = ceil(sum of w / (cap - 1)),
 // a member with w >= tau is planned by G = floor(w / tau) blocks (at most
-// kPlanMaxBlocks; the grid barrier on its own arrival counter, reset at the
+// kPlanMaxBlocks; one if that does, plan_slot_blocks; the grid barrier on its own arrival counter, reset at the
 // end of each launch, so the grid may change from step to step). The others
 // (light) each get a block of their own when the heavy members' blocks and
 // one per light member fit in the launch (a member's plan is mostly latency,
@@ -687,6 +690,17 @@ __device__ __forceinline__ long long plan_slot_work(const SimDev *__restrict__ d
     if (!sc) return -1; // an empty slot
     const long long c = sc->plan_work;
     return (c > 0 ? c : 0) + ds[i].W + kPlanWorkFloor;
+}
+
+// The planner blocks that w of work get at tau each; one for a member whose
+// first pass and front one block does at once without crowding its SM (a
+// second block costs grid barriers: 128 members of 64 to 512 columns, 40 to
+// 300 candidates each, planned by two blocks or mostly by one: 89.4 against 85.5 us per step).
+__device__ __forceinline__ long long plan_slot_blocks(const SimDev *__restrict__ ds, int i, long long w, long long tau)
+{
+    const long long cand = w - ds[i].W - kPlanWorkFloor;
+    if (cand <= PLAN_NT / 2 && ds[i].MW <= PLAN_WARPS) return 1;
+    return min(w / tau, (long long)kPlanMaxBlocks);
 }
 
 template <typename S, typename LT = Lat9>
@@ -709,7 +723,7 @@ __global__ void __launch_bounds__(PLAN_NT, 2) k_plan_batch(const SimDev *__restr
     long long need = 0;
     for (int i = tid; i < nslots; i += PLAN_NT) {
         const long long w = plan_slot_work(ds, i);
-        if (w >= tau) need += w / tau < kPlanMaxBlocks ? w / tau : kPlanMaxBlocks;
+        if (w >= tau) need += plan_slot_blocks(ds, i, w, tau);
         else if (w >= 0) need += 1;
     }
     need = plan_block_sum(need, s_red);
@@ -721,7 +735,7 @@ __global__ void __launch_bounds__(PLAN_NT, 2) k_plan_batch(const SimDev *__restr
         long long hg = 0, lw = 0;
         if (i < nslots) {
             const long long w = plan_slot_work(ds, i);
-            if (w >= tau) hg = w / tau < kPlanMaxBlocks ? w / tau : kPlanMaxBlocks;
+            if (w >= tau) hg = plan_slot_blocks(ds, i, w, tau);
             else if (w >= 0) lw = own ? 1 : w;
         }
         // two exclusive block scans (64-bit: the work sums)
@@ -772,7 +786,7 @@ __global__ void __launch_bounds__(PLAN_NT, 2) k_plan_batch(const SimDev *__restr
             if (s_hpre[mid] <= b) lo = mid; else hi = mid - 1;
         }
         const long long w = plan_slot_work(ds, lo);
-        const int G = (int)(w / tau < kPlanMaxBlocks ? w / tau : kPlanMaxBlocks);
+        const int G = (int)plan_slot_blocks(ds, lo, w, tau);
         plan_body<S, LT>(ds[lo], 0, G, b - s_hpre[lo]);
         return;
     }
@@ -853,6 +867,8 @@ __device__ __forceinline__ void inject_body(const SimDev &d, int blk, int nblk)
 template <typename S, typename LT = Lat9>
 __global__ void k_inject(SimDev d)
 {
+    grid_dependency_wait();   // the planner's selection
+    grid_dependents_launch(); // (the update may start, and wait for this grid)
     inject_body<S, LT>(d, (int)blockIdx.x, (int)gridDim.x);
 }
 

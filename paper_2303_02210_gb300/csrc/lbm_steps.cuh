@@ -615,7 +615,7 @@ __device__ __forceinline__ bool plan_step(const SimDev &d, StepScratch<NT> &ps, 
             if (lr >= 0) {
                 const long long rank = before + lr;
                 if (rank == ns - 1) ps.kstop = (unsigned long long)((long long)blk * C + j + 1);
-                if (rank < ns) plan_select<R, LT>(d, ps.key[j], (int)rank, buf, nyr);
+                if (rank < ns) plan_select<R, true, LT>(d, ps.key[j], (int)rank, buf, nyr);
             }
         }
         acc = total;
@@ -663,7 +663,7 @@ __device__ __forceinline__ bool plan_step(const SimDev &d, StepScratch<NT> &ps, 
                 if (lr < 0) continue;
                 const long long rank = acc + bf + pr + lr;
                 if (rank == ns - 1) ps.kstop = (unsigned long long)(k0 + i + 1);
-                if (rank < ns) plan_select<R, LT>(d, ps.key[tid * kStepR + i], (int)rank, buf, nyr);
+                if (rank < ns) plan_select<R, true, LT>(d, ps.key[tid * kStepR + i], (int)rank, buf, nyr);
             }
             acc += tt;
             base += (long long)G * NT * kStepR;
