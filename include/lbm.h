@@ -244,9 +244,12 @@ int lbm_last_events(lbm_sim *sim, int64_t *node, int32_t *pair, int32_t *count, 
 int lbm_stats(lbm_sim *sim, lbm_stats_t *out);
 
 /* Clears the sticky device status bits, and restarts the planner's grid-
- * barrier counter and division merge table (which hold nothing between steps;
- * after a step abandoned on LBM_STATUS_TIMEOUT they may be inconsistent).
- * Enqueues only. */
+ * barrier counter, its exchanges, its division merge table and the unused ends
+ * of its division lists (which hold nothing between steps; after a step
+ * abandoned on LBM_STATUS_TIMEOUT they may be inconsistent). The divisions of
+ * the latest step (lbm_last_events) and those already selected for the coming
+ * one are kept: a run goes on as it would have without the call. Enqueues
+ * only. */
 int lbm_clear_status(lbm_sim *sim);
 
 /* Failure-detection test hook (no counterpart in the paper). Every wait in

@@ -346,6 +346,19 @@ __global__ void k_export_front(const int32_t *__restrict__ h, const long long *_
     if (blockIdx.x == 0 && threadIdx.x < 2) s_out[threadIdx.x] = s12[threadIdx.x];
 }
 
+// Division counts beyond the selections the two lists hold, the latest step's
+// (n_events) and the coming step's (rec_n): zero, as a launch of many steps
+// relies on.
+__global__ void k_clear_counts(const DevScalars *__restrict__ sc, int32_t *__restrict__ ev_count, int ns_max)
+{
+    const int next = (int)(sc->step & 1); // the coming step's list
+    for (int b = 0; b < 2; ++b) {
+        const int kept = b == next ? sc->rec_n : sc->n_events;
+        for (int r = kept + (int)(blockIdx.x * blockDim.x + threadIdx.x); r < ns_max; r += (int)(gridDim.x * blockDim.x))
+            ev_count[(size_t)b * (size_t)ns_max + (size_t)r] = 0;
+    }
+}
+
 cudaError_t export_front(const lbm_sim *s, int32_t *h_dev, long long *s_dev)
 {
     const int W = s->p.width;
@@ -854,13 +867,15 @@ int lbm_clear_status(lbm_sim *s)
     USE_DEVICE(s);
     CK(cudaMemsetAsync(&s->d.sc->status, 0, sizeof(int), s->stream));
     // after a step abandoned on a timeout the planner's grid-barrier counter
-    // may be off a multiple of its grid and its merge table may hold entries
-    // no list points at: both restart (between steps they hold nothing the
-    // next planner needs)
+    // may be off a multiple of its grid, its merge table may hold entries no
+    // list points at and the count lists entries beyond their selections: all
+    // restart (between steps they hold nothing the next step needs; the counts
+    // of the latest step's divisions and of the coming step's stay)
     CK(cudaMemsetAsync(&s->d.sc->bar_ctr, 0, sizeof(unsigned long long), s->stream));
     CK(cudaMemsetAsync(s->d.htab, 0xFF, (size_t)s->L.hcap * 8u, s->stream));
     CK(cudaMemsetAsync(s->d.xch, 0, kXchBytes, s->stream)); // (a step may be run again under the same number)
-    CK(cudaMemsetAsync(s->d.ev_count, 0, (size_t)s->L.ns_max * 8u, s->stream)); // (zero beyond the current selections)
+    k_clear_counts<<<152, 256, 0, s->stream>>>(s->d.sc, s->d.ev_count, s->L.ns_max);
+    CK(cudaGetLastError());
     return LBM_OK;
 }
 
