@@ -425,8 +425,8 @@ __device__ __forceinline__ bool plan_step(const SimDev &d, StepScratch<NT> &ps, 
         topa = max(topa, ps.top[i]);
         lowa = min(lowa, ps.low[i]);
     }
+    const int Gs = whole ? 1 : min(G, (d.MW + WARPS - 1) / WARPS); // the CTAs whose sums are exchanged
     if (!whole && G > 1) {
-        const int Gs = min(G, (d.MW + WARPS - 1) / WARPS); // the CTAs that have words
         if (tid == 0 && blk < Gs) {
             unsigned long long *x = d.xch + blk * kXch;
             if (d.growth_mode == GROW_EDGE) __threadfence(); // the heights of all this CTA's threads come first
@@ -572,8 +572,9 @@ __device__ __forceinline__ bool plan_step(const SimDev &d, StepScratch<NT> &ps, 
     const size_t buf = (size_t)(tn & 1u) * (size_t)d.ns_max; // event list of step tn
 
     // ---- C/D: candidates in draw order, the first n_s accepted, merged (as
-    // plan_body). Without divisions the counts are still exchanged when
-    // nothing was before: block 0 must not commit while another CTA reads.
+    // plan_body). Without divisions the counts are still exchanged when some
+    // CTA has posted nothing so far (it has no word of the front): block 0 must
+    // not commit while another CTA reads.
     long long acc = 0;
     auto accept = [&](const Candidate &c) -> bool {
         const R rs = rho_star<S, LT>(d, f, nyr, c.x, c.y);
@@ -586,7 +587,7 @@ __device__ __forceinline__ bool plan_step(const SimDev &d, StepScratch<NT> &ps, 
         default: return false;
         }
     };
-    if (ns > 0 || (whole && G > 1)) { // uniform
+    if (ns > 0 || G > Gs) { // uniform
         const long long cap = ns > 0 ? 64 * ns + 1024 : 0;
         int tot_b = 0;
 #pragma unroll 1
