@@ -159,8 +159,14 @@ Layout make_layout(const lbm_params_t &p)
     L.off_evc = o; o = align256(o + (uint64_t)L.ns_max * 8u);
     L.off_rown = o; o = align256(o + (uint64_t)L.ns_max * 4u);
     L.off_rec = o; o = align256(o + (uint64_t)L.ns_max * 8u);
-    L.off_bcnt = o; o = align256(o + (uint64_t)kTmaMaxCtas * 4u);
-    L.off_bucket = o; o = align256(o + (uint64_t)kTmaMaxCtas * kBucketCap * 8u);
+    // division buckets of the staged update's CTAs, which number at most
+    // kTmaMaxCtas and one per eight tiles of the lattice, tiles of two rows
+    // the smallest (lbm_create); none where no form is staged
+    const uint64_t tiles = (uint64_t)((p.width + kTmaBoxX - 1) / kTmaBoxX) * (uint64_t)((p.height + 1) / 2);
+    const bool staged = p.precision != LBM_FP64 && !p.y_periodic;
+    const uint64_t ctas = staged ? std::min<uint64_t>(kTmaMaxCtas, std::max<uint64_t>(2, (tiles + 7) / 8)) : 0;
+    L.off_bcnt = o; o = align256(o + ctas * 4u);
+    L.off_bucket = o; o = align256(o + ctas * kBucketCap * 8u);
     // planner partials: S1, S2, frozen mass (int64); top, low, two count buffers (int32)
     L.off_pl64 = o; o = align256(o + (uint64_t)kPlanMaxBlocks * 3u * 8u);
     L.off_pl32 = o; o = align256(o + (uint64_t)kPlanMaxBlocks * 4u * 4u);

@@ -207,7 +207,7 @@ struct SimDev {
     int upd_tyl2;         // log2 of the rows per tile of the TMA-staged update
     int *rec_owner;       // per division (draw rank): owning CTA of its tile (-1: a repeat)
     unsigned long long *rec; // and its record (pack_record; the amount is ev_count * rho_cell / 2)
-    int *bucket_cnt;      // divisions per CTA of the TMA-staged update (kTmaMaxCtas)
+    int *bucket_cnt;      // divisions per CTA of the TMA-staged update (upd_ctas)
     unsigned long long *bucket; // their records (pack_record), kBucketCap per CTA
     // per-block partials of the fused planner (kPlanMaxBlocks each)
     long long *pl_s1, *pl_s2, *pl_mass;
@@ -308,7 +308,7 @@ int lbm_record_cuda_error(cudaError_t e);
 constexpr int kXO = 4;
 constexpr int kTmaBoxX = 128;
 constexpr int kTmaMaxCtas = 2048; // the reciprocal above is exact for tile * upd_ctas < 2^32
-constexpr int kBucketCap = 256;    // division records listed per update CTA (more: full scan)
+constexpr int kBucketCap = 128;    // division records listed per update CTA, one a thread (more: full scan)
 constexpr int kPlanMaxBlocks = 1024;
 // A launch of many steps (lbm_steps.cuh): planner CTAs, exchanged words of 8
 // bytes per CTA, and steps per launch.

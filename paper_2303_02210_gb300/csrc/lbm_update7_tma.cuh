@@ -222,7 +222,7 @@ __device__ __forceinline__ bool update7_tma_step(const SimDev &d, const CUtensor
         return (float)((double)d.ev_count[(size_t)(t & 1u) * (size_t)d.ns_max + (size_t)e] * d.half_cell);
     };
     // (one entry per thread, read without waiting for their number)
-    static_assert(NT >= TMA_EV_CAP && kBucketCap >= TMA_EV_CAP, "one bucket entry per thread");
+    static_assert(NT >= TMA_EV_CAP, "one bucket entry per thread");
     const unsigned long long rec = d.inject_in_update && tid < TMA_EV_CAP ? d.bucket[blockIdx.x * kBucketCap + tid] : 0ull;
     const int in_bucket = d.inject_in_update ? d.bucket_cnt[blockIdx.x] : 0;
     const int mine = nev_all > 0 ? in_bucket : 0;

@@ -44,7 +44,7 @@ constexpr int TMA_TX = kTmaBoxX;   // 128 columns: two warps of 64
 constexpr int TMA_LX = TMA_TX + 8; // staged columns x0 - 4 .. x0 + 131
 // Divisions of a CTA kept in shared memory (more are read from global memory
 // per tile); tiles flagged per CTA.
-constexpr int TMA_EV_CAP = 128;
+constexpr int TMA_EV_CAP = kBucketCap;
 constexpr int TMA_KFLAG_WORDS = 32;
 static_assert(kXO % 4 == 0, "tile boxes start on 16-byte boundaries");
 
@@ -353,7 +353,7 @@ __device__ __forceinline__ bool update_tma_step(const SimDev &d, const CUtensorM
         return (float)((double)d.ev_count[(size_t)(t & 1u) * (size_t)d.ns_max + (size_t)e] * d.half_cell);
     };
     // (one entry per thread, read without waiting for their number)
-    static_assert(NT >= TMA_EV_CAP && kBucketCap >= TMA_EV_CAP, "one bucket entry per thread");
+    static_assert(NT >= TMA_EV_CAP, "one bucket entry per thread");
     const unsigned long long rec = d.inject_in_update && tid < TMA_EV_CAP ? d.bucket[blockIdx.x * kBucketCap + tid] : 0ull;
     const int in_bucket = d.inject_in_update ? d.bucket_cnt[blockIdx.x] : 0;
     const int mine = nev_all > 0 ? in_bucket : 0;
