@@ -7,8 +7,12 @@
 #include <cstdlib>
 #include <cstring>
 #include <algorithm>
+#include <atomic>
+#include <map>
 #include <mutex>
+#include <new>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include <cudaTypedefs.h>
@@ -304,6 +308,69 @@ bool encode_population_map(CUtensorMap *m, void *base, int nx, int Wp, int H, lo
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// A live simulation's or batch's share of a device: the SMs that its update's
+// grid fills, on its stream. A launch of many steps holds the SMs of its whole
+// grid for all of them, so it pays while the largest grids of all streams fit
+// side by side, and not beyond, where such launches run one after another (and
+// a batch's planners, which fill the device, after them). A step of each of N
+// simulations on streams of their own, two launches a step against one launch of
+// many: 128 x 53 nodes (7 SMs each) N = 8 40.7 against 14.4 us, 1024 x 53 (66
+// SMs) N = 2 28.2 against 16.6, N = 8 30.8 against 62.4, 1024 x 300 (92 SMs)
+// N = 2 28.7 against 43.9, 2048 x 1000 (152) N = 4 116 against 174.
+// Held from creation to destruction, whether or not steps are in flight.
+class StreamShare {
+    using Key = std::pair<int, const void *>; // device, stream
+    struct Ledger {
+        std::mutex lock;
+        std::map<Key, std::map<int, int>> streams; // each stream's shares: SMs -> holders
+        std::atomic<int> total[64] = {};           // of each device: the sum of its streams' largest
+    };
+    static Ledger &ledger()
+    {
+        static Ledger *l = new Ledger; // (outlives every holder)
+        return *l;
+    }
+    Key key{0, nullptr};
+    int sms = 0;
+    bool held = false;
+
+public:
+    StreamShare() = default;
+    StreamShare(const StreamShare &) = delete;
+    StreamShare &operator=(const StreamShare &) = delete;
+    // (a per-thread default stream is another one for every holder)
+    bool take(int device, cudaStream_t stream, int share)
+    {
+        key = {device, stream == cudaStreamPerThread ? (const void *)this
+                       : stream == cudaStreamLegacy ? nullptr : (const void *)stream};
+        sms = share;
+        Ledger &l = ledger();
+        std::lock_guard<std::mutex> g(l.lock);
+        try {
+            std::map<int, int> &m = l.streams[key];
+            const int before = m.empty() ? 0 : m.rbegin()->first;
+            ++m[sms];
+            if (device < 64) l.total[device] += m.rbegin()->first - before;
+            held = true;
+        } catch (const std::bad_alloc &) {
+        }
+        return held;
+    }
+    ~StreamShare()
+    {
+        if (!held) return;
+        Ledger &l = ledger();
+        std::lock_guard<std::mutex> g(l.lock);
+        std::map<int, int> &m = l.streams[key];
+        const int before = m.rbegin()->first;
+        if (--m[sms] == 0) m.erase(sms);
+        if (key.first < 64) l.total[key.first] -= before - (m.empty() ? 0 : m.rbegin()->first);
+        if (m.empty()) l.streams.erase(key);
+    }
+    // whether the grids of all streams of this device (nsm SMs) fit side by side
+    bool alone(int nsm) const { return held && key.first < 64 && ledger().total[key.first] <= nsm; }
+};
+
 } // namespace
 
 int lbm::lbm_record_cuda_error(cudaError_t e) { return cuda_fail(e); }
@@ -324,6 +391,8 @@ struct lbm_sim {
     bool use_tma;
     bool fused;       // many steps in one launch (update_kernel 0),
     bool lone_splits; // but a call of one step as two launches
+    int nsm;          // SMs of the device
+    StreamShare share;
     int tma_grid, tma_variant;
     CUtensorMap maps[4]; // loads from copy 0, 1; stores into copy 0, 1 (variants that store in bulk)
     // kernel timing
@@ -661,6 +730,7 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
     const long long nodes = window_nodes(*p, rows);
     s->lone_splits = lone_step_splits(*p, nodes);
     s->use_tma = s->fused = false;
+    s->nsm = nsm;
     s->tma_grid = nsm;
     // staged update variant (KernelTable::tma_info): "tma" 0 (two-row tiles),
     // "tma1" 1 (four-row tiles), "tma_st" 2 (two-row tiles stored in bulk,
@@ -746,6 +816,8 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
         e = cudaStreamSynchronize(s->stream);
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
     } while (0);
+    const int per_sm = s->use_tma ? ctas_per_sm : std::max(1, bps), grid = s->use_tma ? d.upd_ctas : d.update_grid;
+    if (rc == LBM_OK && !s->share.take(dev, s->stream, std::min(nsm, (grid + per_sm - 1) / per_sm))) rc = LBM_ERR_OOM;
     if (rc != LBM_OK) {
         lbm_destroy(s);
         return rc;
@@ -777,7 +849,7 @@ int lbm_step(lbm_sim *s, int64_t nsteps)
 {
     if (!s || nsteps < 0) return LBM_ERR_INVALID_ARG;
     USE_DEVICE(s);
-    if (s->fused && !s->timing && !(nsteps == 1 && s->lone_splits)) {
+    if (s->fused && !s->timing && !(nsteps == 1 && s->lone_splits) && s->share.alone(s->nsm)) {
         // (launches of at most kStepsPerLaunch steps: work on other streams
         // gets its turn between them)
         for (int64_t left = nsteps; left > 0;) {
@@ -1229,6 +1301,7 @@ struct lbm_batch {
     CUtensorMap *maps;
     int noise, tstore, tma_grid;
     int nsm;
+    StreamShare share; // the whole device (the planners' launch fills it)
     // host copies of the tables
     std::vector<SimDev> h_ds;
     std::vector<int4> h_upd;
@@ -1501,6 +1574,7 @@ cudaError_t batch_init(lbm_batch *b)
         if (e == cudaSuccess) b->branch.push_back(st);
     }
     if (e != cudaSuccess) return e;
+    if (!b->share.take(b->device, b->origin, b->nsm)) return cudaErrorMemoryAllocation;
     if (!b->fused) return batch_recapture(b);
     // the cooperative planner launch: every resident block
     b->plan_cap = std::max(2, b->kt->plan_blocks_per_sm(1) * b->nsm);
