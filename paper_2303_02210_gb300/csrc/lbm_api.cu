@@ -315,8 +315,8 @@ bool encode_population_map(CUtensorMap *m, void *base, int nx, int Wp, int H, lo
 // a batch's planners, which fill the device, after them). A step of each of N
 // simulations on streams of their own, two launches a step against one launch of
 // many: 128 x 53 nodes (7 SMs each) N = 8 40.7 against 14.4 us, 1024 x 53 (66
-// SMs) N = 2 28.2 against 16.6, N = 8 30.8 against 62.4, 1024 x 300 (92 SMs)
-// N = 2 28.7 against 43.9, 2048 x 1000 (152) N = 4 116 against 174.
+// SMs) N = 2 28.2 against 16.6, N = 8 30.3 against 62.4, 1024 x 300 (92 SMs)
+// N = 2 29.3 against 43.9, 2048 x 1000 (152) N = 4 111 against 174.
 // Held from creation to destruction, whether or not steps are in flight.
 class StreamShare {
     using Key = std::pair<int, const void *>; // device, stream
