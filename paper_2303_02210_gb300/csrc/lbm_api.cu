@@ -253,21 +253,34 @@ long long window_nodes(const lbm_params_t &p, const std::vector<int32_t> &rows0)
     return (std::min<long long>(p.height, top + 2) - rear) * p.width;
 }
 
-// Whether steps run many to a launch (lbm_steps.cuh) rather than as two
-// launches each: while the step's fixed cost counts. By the window's nodes, us
-// per step in one launch against two: FP32 23 against 27 at 0.5M nodes, 44 / 47
-// at 2.1M, 70.0 / 71.5 at 4.2M (as long over 20 steps, with the launch),
-// 118.6 / 117.2 at 8.4M (a lone update then has fewer spills and the planner's
-// share is small); 16 bits, which are bound by their instructions, 43.4 / 45.7
-// at 2.1M, 73.2 / 72.3 at 4.2M, 118.4 / 114.0 at 8.4M; D2Q7 63.5 / 65.2 at 4.2M,
+// The fewest steps of one call that run many to a launch (lbm_steps.cuh) rather
+// than as two launches each; 0 if none. `nodes`: the initial window's.
+//
+// Long calls take the form while a step's fixed cost counts. Us per step in
+// one launch against two: FP32 20.0 / 24.7 at 0.3M nodes, 29.9 / 32.6 at 1M, 43.3
+// / 47.1 at 2M, 58.2 / 59.4 at 2.9M, 70.0 / 71.5 at 4.2M (as long over 20 steps,
+// with the launch), 118.6 / 117.2 at 8.4M (a lone update has no spills, and the
+// planner's share is small). 16 bits, bound by their instructions: 30.2 / 32.8 at
+// 1M, 41.8 / 45.0 at 2M, 53.7 / 51.0 at 2.5M, 55.6 / 57.5 at 2.9M, 73.2 / 72.3
+// at 4.2M. D2Q7 27.8 / 30.8 at 1M, 51.5 / 51.9 at 2.9M, 63.5 / 65.2 at 4.2M,
 // 105.6 / 109.6 at 8.4M.
-bool fused_pays(const lbm_params_t &p, long long nodes) { return p.lattice == LBM_D2Q7 || nodes <= 3ll << 20; }
-
-// Whether a call of a single step takes the two launches all the same: they
-// overlap with the launches around them (programmatic dependents), which a
-// cooperative launch does not. Single steps of 2048 x 512 nodes 33.6 us against
-// 35.2, of 1024 x 256 24.3 against 25.2, of 512 x 52 21.3 against 19.3.
-bool lone_step_splits(const lbm_params_t &p, long long nodes) { return p.lattice == LBM_D2Q9 && nodes >= 1ll << 19; }
+//
+// Short calls take the two launches, which overlap with the launches around
+// them (programmatic dependents), where a cooperative launch waits for the
+// stream to drain, about 4.5 us a call: FP32 n = 1 20.5 / 22.6 at 152k nodes but
+// 22.8 / 21.7 at 207k and 27.4 / 24.6 at 225k; n = 2 21.1 / 21.6 at 207k, 27.7 /
+// 26.7 at 0.53M; n = 4 24.2 / 26.6 at 0.5M, 28.7 / 28.5 at 0.64M in 16 bits, 36.0
+// / 34.9 at 1.2M; n = 8 35.3 / 34.9 there, 48.2 / 52.5 at 2.25M, 54.0 / 54.8 at
+// 2.5M; D2Q7 n = 4 30.9 / 32.8 at 1.2M, 35.4 / 35.0 at 1.4M, 52.7 / 52.1 at 2.9M.
+int64_t fused_min_steps(const lbm_params_t &p, long long nodes)
+{
+    const bool d2q7 = p.lattice == LBM_D2Q7;
+    const long long most = p.precision == LBM_FP32 ? 3ll << 20 : 2ll << 20;
+    if (!d2q7 && nodes > most) return 0;
+    if (nodes < 3ll << 16) return 1;
+    if (nodes < 1ll << 18) return 2;
+    return d2q7 || nodes < 1ll << 20 ? 4 : 8;
+}
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no
 // link-time dependency on the driver library).
@@ -389,8 +402,7 @@ struct lbm_sim {
     int64_t launches;
     // TMA-staged update (FP32, walls in y)
     bool use_tma;
-    bool fused;       // many steps in one launch (update_kernel 0),
-    bool lone_splits; // but a call of one step as two launches
+    int64_t fused_steps; // a call of at least so many steps runs many to a launch (0: none)
     int nsm;          // SMs of the device
     StreamShare share;
     int tma_grid, tma_variant;
@@ -728,8 +740,8 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
     std::vector<int32_t> rows;
     front_rows(*p, rows);
     const long long nodes = window_nodes(*p, rows);
-    s->lone_splits = lone_step_splits(*p, nodes);
-    s->use_tma = s->fused = false;
+    s->use_tma = false;
+    s->fused_steps = 0;
     s->nsm = nsm;
     s->tma_grid = nsm;
     // staged update variant (KernelTable::tma_info): "tma" 0 (two-row tiles),
@@ -790,8 +802,9 @@ int lbm_create(const lbm_params_t *p, void *stream, void *arena, uint64_t arena_
             s->use_tma = false;
             d.inject_in_update = 0;
         }
-        s->fused = s->use_tma && p->update_kernel == 0 && s->kt->tma_steps && fused_pays(*p, nodes) &&
-                   s->kt->tma_steps(d, nullptr, variant, 0, s->stream) == cudaSuccess;
+        if (s->use_tma && p->update_kernel == 0 && s->kt->tma_steps &&
+            s->kt->tma_steps(d, nullptr, variant, 0, s->stream) == cudaSuccess)
+            s->fused_steps = fused_min_steps(*p, nodes);
         if (!ok && p->update_kernel >= 2 && p->update_kernel != 5) {
             if (s->own_arena) cudaFree(s->arena);
             delete s;
@@ -849,7 +862,7 @@ int lbm_step(lbm_sim *s, int64_t nsteps)
 {
     if (!s || nsteps < 0) return LBM_ERR_INVALID_ARG;
     USE_DEVICE(s);
-    if (s->fused && !s->timing && !(nsteps == 1 && s->lone_splits) && s->share.alone(s->nsm)) {
+    if (s->fused_steps && nsteps >= s->fused_steps && !s->timing && s->share.alone(s->nsm)) {
         // (launches of at most kStepsPerLaunch steps: work on other streams
         // gets its turn between them)
         for (int64_t left = nsteps; left > 0;) {
