@@ -337,6 +337,7 @@ class StreamShare {
         std::mutex lock;
         std::map<Key, std::map<int, int>> streams; // each stream's shares: SMs -> holders
         std::atomic<int> total[64] = {};           // of each device: the sum of its streams' largest
+        std::atomic<unsigned> emptied[64] = {};    // times a device's last holder went
     };
     static Ledger &ledger()
     {
@@ -379,7 +380,9 @@ public:
         if (--m[sms] == 0) m.erase(sms);
         if (key.first < 64) l.total[key.first] -= before - (m.empty() ? 0 : m.rbegin()->first);
         if (m.empty()) l.streams.erase(key);
+        if (key.first < 64 && l.total[key.first] == 0) ++l.emptied[key.first];
     }
+    static unsigned emptied(int device) { return device < 64 ? ledger().emptied[device].load() : 0u; }
     // whether the grids of all streams of this device (nsm SMs) fit side by side
     bool alone(int nsm) const { return held && key.first < 64 && ledger().total[key.first] <= nsm; }
 };
@@ -474,17 +477,42 @@ void *device_alias(void *p)
     return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+// The process-wide unique number of the allocation that p lies in, 0 if none
+// (freed, or gone with its context in a cudaDeviceReset).
+unsigned long long buffer_id(void *p)
+{
+    static const PFN_cuPointerGetAttribute_v4000 get = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return (PFN_cuPointerGetAttribute_v4000)fn;
+    }();
+    unsigned long long id = 0;
+    return get && get(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, (CUdeviceptr)p) == CUDA_SUCCESS ? id : 0;
+}
+
 // A block of pinned host memory (two sums and the widest front) for the
 // duration of one call. Blocks are kept for later calls, kStagingKept at most
-// (about 1 MB in all); a call that finds none allocates its own and frees it
-// if enough are kept. Any thread, any device (portable); null (the caller then
-// copies) if the memory cannot be had.
+// (about 1 MB in all, for the life of the process: an allocation and its release
+// take 290 us, more than the rest of a short run from create to destroy); a call
+// that finds none allocates its own and frees it if enough are kept. A block
+// that a device reset has taken (between the simulations of its device) is told
+// by its number and dropped. Any thread, any device (portable); null (the caller
+// then copies) if the memory cannot be had.
 class StagingLease {
     static constexpr size_t kBytes = 2 * sizeof(long long) + 32768 * sizeof(int32_t);
     static constexpr int kStagingKept = 8;
+    struct Block {
+        char *p;
+        unsigned long long id;
+        int device;    // current when it was allocated
+        unsigned seen; // StreamShare::emptied of it when the block was last in use
+    };
     struct Kept {
         std::mutex lock;
-        char *blocks[kStagingKept];
+        Block blocks[kStagingKept];
         int n = 0;
     };
     static Kept &kept()
@@ -492,43 +520,46 @@ class StagingLease {
         static Kept k;
         return k;
     }
-    char *p = nullptr;
+    Block b{nullptr, 0, 0, 0};
 
 public:
-    StagingLease()
+    explicit StagingLease(int device)
     {
         {
             std::lock_guard<std::mutex> g(kept().lock);
-            if (kept().n > 0) {
-                p = kept().blocks[--kept().n];
-                return;
+            while (kept().n > 0) {
+                b = kept().blocks[--kept().n];
+                if (b.seen == StreamShare::emptied(b.device) || buffer_id(b.p) == b.id) return;
             }
         }
+        b = Block{nullptr, 0, 0, 0};
         void *q = nullptr;
         if (cudaHostAlloc(&q, kBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
             cudaGetLastError();
             return;
         }
-        if (device_alias(q) == q) // (unified addressing)
-            p = (char *)q;
+        const unsigned long long id = device_alias(q) == q ? buffer_id(q) : 0; // (unified addressing)
+        if (id)
+            b = Block{(char *)q, id, device, 0};
         else
             cudaFreeHost(q);
     }
     ~StagingLease()
     {
-        if (!p) return;
+        if (!b.p) return;
+        b.seen = StreamShare::emptied(b.device);
         {
             std::lock_guard<std::mutex> g(kept().lock);
             if (kept().n < kStagingKept) {
-                kept().blocks[kept().n++] = p;
+                kept().blocks[kept().n++] = b;
                 return;
             }
         }
-        cudaFreeHost(p);
+        cudaFreeHost(b.p);
     }
     StagingLease(const StagingLease &) = delete;
     StagingLease &operator=(const StagingLease &) = delete;
-    char *get() const { return p; }
+    char *get() const { return b.p; }
 };
 
 } // namespace
@@ -988,7 +1019,7 @@ int lbm_front_heights(lbm_sim *s, int32_t *h_host, double *hbar, double *w)
 {
     if (!s) return LBM_ERR_INVALID_ARG;
     USE_DEVICE(s);
-    if (StagingLease lease; lease.get()) {
+    if (StagingLease lease(s->device); lease.get()) {
         // through pinned memory that the device writes itself: one small launch
         // and a host copy instead of two copies into pageable memory (a step
         // and its front of the 128-column lattice: 39.7 -> 27.7 us)
