@@ -45,9 +45,10 @@ __host__ __device__ __forceinline__ int key_y(uint32_t k) { return (int)(k >> 17
 __host__ __device__ __forceinline__ int key_pair(uint32_t k) { return (int)(k & 3u); }
 
 // A division's record in its update CTA's bucket: draw rank (< 2^24), the
-// tile's index among the CTA's tiles (at most 2^30 nodes in tiles of 256 over
-// at least an eighth as many CTAs or all that fit: < 2^14) and the two staged
-// offsets (< 2^13).
+// tile's index among the CTA's tiles (kTilesPerCta bounds it: the largest
+// lattice has 5519 a CTA on 152 SMs; a lattice with more, on a fraction of the
+// device, is not staged) and the two staged offsets (< 2^13).
+constexpr int kTilesPerCta = 1 << 14;
 __host__ __device__ __forceinline__ unsigned long long pack_record(int rank, int k, int off0, int off1)
 {
     return (unsigned long long)(uint32_t)rank << 40 | (unsigned long long)(uint32_t)k << 26 |
