@@ -10,8 +10,9 @@
 // what does not depend on the update (the candidates' Philox blocks, the
 // pending statistics) is done before it ends. Per step, two launches against
 // one: 128 columns by 53 rows 20.5 -> 13.0 us, 1024 by 53 20.5 -> 15.7, 1501 by
-// 53 in BF16 23.1 -> 17.6, 1024 by 512 26.7 -> 23.1, 4096 by 1003 72.7 -> 70.3,
-// D2Q7 4096 by 1003 66.2 -> 63.8. What is left at 128 columns: four hand-overs
+// 53 in BF16 23.1 -> 17.6, 1024 by 490 26.1 -> 23.3, 2048 by 976 47.1 -> 43.5,
+// D2Q7 4096 by 1003 66.2 -> 63.8 (which calls take it: fused_min_steps in
+// lbm_api.cu). What is left at 128 columns: four hand-overs
 // between CTAs of about 1 us each, the front's scan 0.9, the candidates'
 // gathers 1.0, the divisions' atomics 1.6, the update itself 2.5.
 //
