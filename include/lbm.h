@@ -176,7 +176,7 @@ int lbm_create(const lbm_params_t *params, void *stream, void *arena, uint64_t a
  * heights, Eq. 6 width, rear wall and active mass), all on the device with no
  * host synchronisation. With update_kernel 0 and an initial active window up to
  * a few million nodes (D2Q7: any), up to 64 steps are one cooperative launch (a
- * call of fewer than 2 to 8 steps only for small windows) as long as the update grids of
+ * call of a few steps only for smaller windows) as long as the update grids of
  * the live simulations and batches of the device, the largest of each stream,
  * fit on it side by side; otherwise, and in kernel timing, a step is an update
  * and a planner launch.
