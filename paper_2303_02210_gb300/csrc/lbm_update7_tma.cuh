@@ -237,10 +237,8 @@ __device__ __forceinline__ bool update7_tma_step(const SimDev &d, const CUtensor
         }
         if (tid == 0) s_nev = mine;
     } else {
-        for (int e = tid; e < nev_all; e += NT) {
-            if (d.rec_owner[e] != (int)blockIdx.x) continue;
+        owned_records<NT>(d.rec_owner, d.rec, nev_all, [&](int e, unsigned long long r) {
             const int at = atomicAdd(&s_nev, 1);
-            const unsigned long long r = d.rec[e];
             const int k = rec_tile(r);
             if (at < TMA_EV_CAP) {
                 ev_k[at] = k;
@@ -249,7 +247,7 @@ __device__ __forceinline__ bool update7_tma_step(const SimDev &d, const CUtensor
                 ev_add[at] = amount(e);
             }
             if (k < 32 * TMA_KFLAG_WORDS) atomicOr(&kflag[k >> 5], 1u << (k & 31));
-        }
+        });
     }
     __syncthreads();
     if (FUSED) {
@@ -290,7 +288,7 @@ __device__ __forceinline__ bool update7_tma_step(const SimDev &d, const CUtensor
         // divisions of this tile, added to the staged pre-stream slots
         // (distinct records never share a slot)
         const bool has_ev =
-            nev > 0 && (ev_overflow || k >= 32 * TMA_KFLAG_WORDS || ((kflag[k >> 5] >> (k & 31)) & 1u));
+            nev > 0 && (k >= 32 * TMA_KFLAG_WORDS || ((kflag[k >> 5] >> (k & 31)) & 1u));
         if (has_ev) { // uniform across the CTA
             if (!ev_overflow) {
                 for (int i = tid; i < nev; i += NT)
@@ -299,12 +297,12 @@ __device__ __forceinline__ bool update7_tma_step(const SimDev &d, const CUtensor
                         stage[ev_off[2 * i + 1]] = stage[ev_off[2 * i + 1]] + ev_add[i];
                     }
             } else {
-                for (int e = tid; e < nev_all; e += NT)
-                    if (d.rec_owner[e] == (int)blockIdx.x && rec_tile(d.rec[e]) == k) {
-                        const float a = amount(e);
-                        stage[rec_off0(d.rec[e])] = stage[rec_off0(d.rec[e])] + a;
-                        stage[rec_off1(d.rec[e])] = stage[rec_off1(d.rec[e])] + a;
-                    }
+                owned_records<NT>(d.rec_owner, d.rec, nev_all, [&](int e, unsigned long long r) {
+                    if (rec_tile(r) != k) return;
+                    const float a = amount(e);
+                    stage[rec_off0(r)] = stage[rec_off0(r)] + a;
+                    stage[rec_off1(r)] = stage[rec_off1(r)] + a;
+                });
             }
             fence_proxy_async_smem(); // before a later bulk copy overwrites them
             __syncthreads();

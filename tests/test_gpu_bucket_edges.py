@@ -28,3 +28,26 @@ def test_buckets_full_and_over(lattice, kernel, per_cta):
         assert np.array_equal(x, y)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("lattice,kernel", [("d2q9", "auto"), ("d2q9", "tma"), ("d2q9", "tma1"), ("d2q9", "tma_st"),
+                                            ("d2q7", "auto"), ("d2q7", "tma")])
+@pytest.mark.parametrize("precision", ["fp32", "fp16"])
+def test_over_in_tiles_at_the_front_alone(lattice, kernel, precision):
+    from paper_2303_02210_gb300.lbm import Simulation
+    if precision == "fp16" and (lattice == "d2q7" or kernel == "tma_st"):
+        pytest.skip("no such form")
+    # 122 tiles of 128 x 2 nodes over 28 CTAs, about ten of them at the front
+    # with 200 divisions each: a CTA over its bucket has tiles without any
+    p = wl.base_params(width=256, height=220, front_row=120.0, growth_mode="edge", edge_depth=8, wall_mode="fixed",
+                       growth_rate=2000 * 0.1 / (256 * 120), lattice=lattice, seed=13)
+    a = Simulation(p, precision=precision, update_kernel="plain")
+    b = Simulation(p, precision=precision, update_kernel=kernel)
+    a.step(8)
+    b.step(8)
+    assert a.stats()["events_last"] >= 1900
+    assert np.array_equal(a.pops(), b.pops())
+    for x, y in zip(a.last_events(), b.last_events()):
+        assert np.array_equal(x, y)
+    a.close()
+    b.close()
