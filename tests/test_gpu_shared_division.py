@@ -1,6 +1,6 @@
 """``SharedDiv`` by itself against IEEE division (NumPy's): random operands,
 quotients next to the midpoint of two numbers, and the ends of the ranges that
-the method takes (the significand 2^-8 short of 2, the smallest and largest
+the method takes (significands just short of 2, the smallest and largest
 divisors and numerators, zeros of either sign), in both widths. What it does not
 take, it must refuse."""
 import ctypes
@@ -59,7 +59,7 @@ def lib(tmp_path_factory):
 
 
 def operands(dtype):
-    p, top, blo, bhi, alo, ahi = (24, 0x7F0000, -30, 30, -60, 60) if dtype is np.float32 else \
+    p, top, blo, bhi, alo, ahi = (24, 0x7FFF00, -30, 30, -60, 60) if dtype is np.float32 else \
         (53, 0xFE000 << 32, -100, 100, -500, 500)
     rng = np.random.default_rng(5)
     n = 1 << 20
@@ -73,6 +73,11 @@ def operands(dtype):
     q = (rng.integers(one, 2 * one, n).astype(np.longdouble) + np.longdouble(0.5)) / np.longdouble(one)
     a.append((sb.astype(np.longdouble) * q).astype(dtype))
     b.append(sb)
+    # the same by divisors just short of 2 (times a power of two)
+    near = np.ldexp((one + rng.integers(top - (1 << (p - 7)), top, n)).astype(dtype) / dtype(one),
+                    rng.integers(blo, bhi, n)).astype(dtype)
+    a.append((near.astype(np.longdouble) * q).astype(dtype))
+    b.append(near)
     # edges
     edge_b = [np.ldexp(dtype(one + m) / dtype(one), e).astype(dtype) for e in (blo, -1, 0, bhi - 1)
               for m in (0, 1, top - 2, top - 1, top, top + 1, one - 1)]
@@ -103,6 +108,6 @@ def test_quotients_are_ieee(lib, dtype):
     p = ctypes.c_void_p
     assert fn(p(a.ctypes.data), p(b.ctypes.data), p(q.ctypes.data), p(taken.ctypes.data), a.size) == 0
     assert np.array_equal(taken.astype(bool), takes)
-    assert takes.sum() > 1.9e6
+    assert takes.sum() > 2.9e6
     u = np.uint32 if dtype is np.float32 else np.uint64
     assert np.array_equal(q[takes].view(u), (a[takes] / b[takes]).view(u))
