@@ -269,18 +269,19 @@ long long window_nodes(const lbm_params_t &p, const std::vector<int32_t> &rows0)
 // launches around them (programmatic dependents), where a cooperative launch
 // waits for the stream to drain, about 4.5 us a call. Calls one after another:
 // FP32 n = 1 20.5 / 22.6 at 152k nodes but 22.8 / 21.7 at 207k and 27.4 / 24.6 at
-// 225k, D2Q7 24.6 / 24.0 at 225k and 28.7 / 25.2 at 0.53M; FP32 n = 2 24.3 / 25.3
-// at 0.41M, 30.9 / 29.0 at 0.82M, 43.3 / 41.2 at 1.6M, D2Q7 26.5 / 25.1 at 0.53M,
-// 37.5 / 37.2 at 1.6M; FP32 n = 4 36.0 / 34.9 at 1.2M, 48.7 / 52.4 at 2.25M, 54.6
-// / 54.8 at 2.5M, 16 bits 39.2 / 37.8 at 1.4M, n = 8 38.8 / 37.4 there. A call
-// whose result is waited for has no launches around it, and one launch starts
-// sooner than several: a step and its front FP32 32.7 / 36.4 at 207k nodes, two
-// 61.5 / 67.9 at 0.53M, 69.3 / 71.6 at 0.82M, 97.1 / 95.2 at 1.6M.
+// 225k, D2Q7 24.6 / 24.0 at 225k, 32.9 / 29.2 at 281k with a rough front and 28.7 /
+// 25.2 at 0.53M; FP32 n = 2 24.3 / 25.3 at 0.41M, 30.9 / 29.0 at 0.82M, 43.3 /
+// 41.2 at 1.6M, D2Q7 26.5 / 25.1 at 0.53M, 37.5 / 37.2 at 1.6M; FP32 n = 4 36.0 /
+// 34.9 at 1.2M, 48.7 / 52.4 at 2.25M, 54.6 / 54.8 at 2.5M, 16 bits 39.2 / 37.8 at
+// 1.4M, n = 8 38.8 / 37.4 there. A call whose result is waited for has no
+// launches around it, and one launch starts sooner than several: a step and its
+// front FP32 32.7 / 36.4 at 207k nodes, two 61.5 / 67.9 at 0.53M, 69.3 / 71.6 at
+// 0.82M, 97.1 / 95.2 at 1.6M.
 int64_t fused_min_steps(const lbm_params_t &p, long long nodes)
 {
     const bool d2q7 = p.lattice == LBM_D2Q7, half = p.precision == LBM_FP16 || p.precision == LBM_BF16;
     if (!d2q7 && nodes > (half ? 2ll << 20 : 3ll << 20)) return 0;
-    if (nodes < (d2q7 ? 3ll << 17 : 3ll << 16)) return 1;
+    if (nodes < (d2q7 ? 1ll << 18 : 3ll << 16)) return 1;
     if (d2q7 || nodes < 1ll << 20) return 2;
     return half ? 8 : 4;
 }
