@@ -40,7 +40,8 @@ namespace lbm {
 
 constexpr int kStepSleep = 100;    // ns between polls of the CTAs that wait for the planner
 constexpr int kStepR = 8;          // candidates per thread in the first pass
-constexpr int kStepWords = 4;      // mask words per warp up to which every planner CTA scans the whole front
+constexpr int kStepWords = 4;      // mask words per warp up to which every planner CTA scans the whole front,
+constexpr int kStepRough = 96;     // and rows of the front
 
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
@@ -170,17 +171,22 @@ __device__ __forceinline__ bool xch_get2(const SimDev &d, int blk, int word, uin
 
 // Planner CTAs of a step (at most kStepMaxPlan), from the number of candidates
 // that the selection before needed (an estimate): 16 candidates a CTA, up to
-// 128 when there are many. A candidate gathers 9 (7) scattered populations and a division does three
-// scattered atomics and stores, and an SM sends such requests at one per
-// several clocks (72 candidates in one CTA: 4300 clocks), so few are spread
-// thin; but every CTA reads every other's counts. A front of more than kStepWords words per warp is scanned by as many
-// CTAs as it has words per warp, and their sums are exchanged; a narrower one
-// by every planner CTA whole (no exchange).
+// 128 when there are many. A candidate gathers 9 (7) scattered populations and a
+// division does three scattered atomics and stores, and an SM sends such
+// requests at one per several clocks (72 candidates in one CTA: 4300 clocks), so
+// few are spread thin; but every CTA reads every other's counts. A front of more
+// than kStepWords words per warp is scanned by as many CTAs as it has words per
+// warp, and their sums are exchanged; a narrower one by every planner CTA whole
+// (no exchange), unless a warp has several words of it and it spans more than
+// kStepRough rows, each 32 of which cost a round for each word (405 columns, 800
+// rows: 48.3 us a step scanned whole, 33.4 exchanged, 44 as two launches; 200
+// rows 23.8 and 21.8; 100 rows 17.6 whole).
 template <int NT>
-__device__ __forceinline__ int step_planners(long long kc, int MW, int ctas, bool *whole)
+__device__ __forceinline__ int step_planners(const DevScalars *sc, int MW, int ctas, bool *whole)
 {
     constexpr int WARPS = NT / 32;
-    *whole = MW <= WARPS * kStepWords;
+    const long long kc = sc->plan_kc;
+    *whole = MW <= WARPS * kStepWords && (MW <= WARPS || sc->H_top - sc->hmin <= kStepRough);
     const long long per = min(max(kc / 64, 16ll), 128ll);
     int G = (int)min((kc + per - 1) / per, (long long)kStepMaxPlan);
     if (!*whole) G = max(G, min((MW + WARPS - 1) / WARPS, kStepMaxPlan));

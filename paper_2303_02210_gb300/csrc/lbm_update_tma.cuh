@@ -314,7 +314,7 @@ __device__ __forceinline__ bool update_tma_step(const SimDev &d, const CUtensorM
     st.budget = budget;
     if (FUSED) {
         st.extra = (d.sc->wait_test & WAIT_TEST_BARRIER) ? 1 : 0;
-        st.G = step_planners<NT>(d.sc->plan_kc, d.MW, (int)gridDim.x, &st.whole);
+        st.G = step_planners<NT>(d.sc, d.MW, (int)gridDim.x, &st.whole);
     }
     const int cur = (int)(t & 1u);
     const CUtensorMap *tm = cur ? tm1 : tm0;
