@@ -277,10 +277,19 @@ long long window_nodes(const lbm_params_t &p, const std::vector<int32_t> &rows0)
 // launches around it, and one launch starts sooner than several: a step and its
 // front FP32 32.7 / 36.4 at 207k nodes, two 61.5 / 67.9 at 0.53M, 69.3 / 71.6 at
 // 0.82M, 97.1 / 95.2 at 1.6M.
+//
+// With a division or more per 400 nodes and step, the planner, which the
+// many-step form spreads over more CTAs, outweighs that: n = 2, D2Q9 FP32 edge
+// growth from a rough front at g = 1e-3 0.24 of the two launches' time at 0.26M
+// nodes, 0.85 at 0.82M and 0.94 at 1.2M, density growth 0.46, 0.89 and 0.97, 16
+// bits 0.85, 0.73 and 0.92 (and 0.27 for edge growth at 3e-3 in a window of 2.8M
+// nodes); n = 1, D2Q7 density growth 0.94, 0.87 and 0.89.
 int64_t fused_min_steps(const lbm_params_t &p, long long nodes)
 {
     const bool d2q7 = p.lattice == LBM_D2Q7, half = p.precision == LBM_FP16 || p.precision == LBM_BF16;
-    if (!d2q7 && nodes > (half ? 2ll << 20 : 3ll << 20)) return 0;
+    const bool growing = p.growth_mode != LBM_GROW_NONE && 400.0 * p.growth_rate * p.rho_init > p.rho_cell;
+    if (!d2q7 && nodes > (half && !growing ? 2ll << 20 : 3ll << 20)) return 0;
+    if (growing) return d2q7 || nodes < 1ll << 19 ? 1 : 2;
     if (nodes < (d2q7 ? 1ll << 18 : 3ll << 16)) return 1;
     if (d2q7 || nodes < 1ll << 20) return 2;
     return half ? 8 : 4;
