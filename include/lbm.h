@@ -179,14 +179,14 @@ int lbm_create(const lbm_params_t *params, void *stream, void *arena, uint64_t a
  * call of a few steps only for smaller windows) as long as the update grids of
  * the live simulations and batches of the device, the largest of each stream,
  * fit on it side by side; otherwise, and in kernel timing, a step is an update
- * and a planner launch.
- * The results are the same bit for bit. Returns LBM_OK or a launch error; device-side status
- * (LBM_STATUS_*) is reported by lbm_stats. */
+ * and a planner launch. The results are the same bit for bit. Returns LBM_OK or
+ * a launch error; device-side status (LBM_STATUS_*) is reported by lbm_stats. */
 int lbm_step(lbm_sim *sim, int64_t nsteps);
 
 /* Front heights h(x) = 1 + highest occupied row of column x (0 if none) into
  * the caller's host array of W int32, and the mean height and interface width
- * w of Eq. 6 (either pointer may be NULL). Syncs. */
+ * w of Eq. 6 (either pointer may be NULL). Keeps up to 8 pinned blocks of
+ * 128 KB for the process's later calls. Syncs. */
 int lbm_front_heights(lbm_sim *sim, int32_t *h_host, double *hbar, double *w);
 
 /* The same without waiting: enqueues on the simulation's stream the copies of
